@@ -11,6 +11,7 @@
 #include <vector>
 
 #include "device.h"
+#include "fixed.h"
 #include "internal.h"
 
 using namespace cteno;
@@ -43,6 +44,8 @@ struct cteno_ctx {
   int hrec = 0, hms = 0;
   uint32_t *cinfo = nullptr, *fmeta = nullptr;
   void *Pc = nullptr, *Pd = nullptr, *Uf = nullptr;
+  int8_t *Pe = nullptr;              // FP64 path, conserved variables: block exponents of Pc, Pd
+  int32_t *phifx = nullptr;          //   and the face table
   uint8_t *flags = nullptr;
   double *geo = nullptr, *vol = nullptr, *dt = nullptr;
   float *geo32 = nullptr;
@@ -125,6 +128,9 @@ KArgs make_args(cteno_ctx *ctx, int stage, int dt_swap) {
   a.cinfo = ctx->cinfo;
   a.Pc = ctx->Pc;
   a.Pd = ctx->Pd;
+  a.Pe = ctx->Pe;
+  a.phifx = (const int2 *)ctx->phifx;
+  for (int k = 0; k < kMaxNK; ++k) a.phi_exp[k] = ctx->tab.phi_exp[k];
   a.Uf = ctx->Uf;
   a.flags = ctx->record_flags ? ctx->flags : nullptr;
   a.nbr = ctx->nbr;
@@ -540,8 +546,21 @@ int cteno_lsq_build(cteno_ctx *ctx) {
   CK(dalloc(ctx, &ctx->nbr, sizeof(int32_t) * 4 * N));
   CK(dalloc(ctx, &ctx->cinfo, sizeof(uint32_t) * N));
   CK(dalloc(ctx, &ctx->fmeta, sizeof(uint32_t) * N));
-  CK(dalloc(ctx, &ctx->Pc, sT * ctx->nk * M * N));
+  const bool fixed = !ctx->fp32 && !ctx->p.characteristic;  // operators as integers (fixed.h)
+  CK(dalloc(ctx, &ctx->Pc, sT * ctx->nk * M * (fixed ? fixed_cells(d, N) : N)));
   CK(dalloc(ctx, &ctx->Pd, sT * nf * pds * N));
+  std::vector<int32_t> hphi;  // the face table, rows of an even number of entries
+  if (fixed) {
+    const int np = d == 3 ? 6 : 1, nkp = (ctx->nk + 1) / 2 * 2;
+    for (int f = 0; f < nf; ++f)
+      for (int p = 0; p < np; ++p)
+        for (int q = 0; q < ctx->nq; ++q)
+          for (int k = 0; k < nkp; ++k)
+            for (int t = 0; t < 2; ++t) hphi.push_back(k < ctx->nk ? tab.PhiFx[f][p][q][k][t] : 0);
+    CK(dalloc(ctx, &ctx->Pe, (size_t)kFixExp * N));
+    CK(dalloc(ctx, &ctx->phifx, hphi.size() * sizeof(int32_t)));
+    CK(cudaMemcpyAsync(ctx->phifx, hphi.data(), hphi.size() * sizeof(int32_t), cudaMemcpyHostToDevice, ctx->stream));
+  }
   CK(dalloc(ctx, &ctx->Uf, sT * nf * ctx->nq * ctx->nv * N));
   CK(dalloc(ctx, &ctx->geo, sizeof(double) * nf * 4 * N));
   if (ctx->fp32) CK(dalloc(ctx, &ctx->geo32, sizeof(float) * nf * 4 * N));
@@ -573,6 +592,7 @@ int cteno_lsq_build(cteno_ctx *ctx) {
   std::memcpy(dt.psibar, tab.psibar, sizeof(dt.psibar));
   std::memcpy(dt.O, tab.O, sizeof(dt.O));
   std::memcpy(dt.Phi, tab.Phi, sizeof(dt.Phi));
+  std::memcpy(dt.LT, tab.LT, sizeof(dt.LT));
   std::memcpy(dt.fw, tab.fw, sizeof(dt.fw));
   std::memcpy(dt.vq, tab.vq, sizeof(dt.vq));
   std::memcpy(dt.vw, tab.vw, sizeof(dt.vw));
@@ -604,6 +624,7 @@ int cteno_lsq_build(cteno_ctx *ctx) {
   for (int j = 0; j < 3; ++j) s.period[j] = 0.0;
   s.Pc = ctx->Pc;
   s.Pd = ctx->Pd;
+  s.Pe = ctx->Pe;
   s.store_fp32 = ctx->fp32 ? 1 : 0;
   s.geo = ctx->geo;
   s.vol = ctx->vol;
@@ -1049,6 +1070,7 @@ int cteno_autotune(cteno_ctx *ctx, int32_t *best_out) {
   // the lane schedules (variable per lane for the reconstruction, face per lane for the flux)
   for (int b : {128, 256}) cand.push_back(kLaneSchedule + b);
   std::vector<int> rcand = cand;
+  if (!ctx->fp32) rcand = {64, 128, 256};  // the FP64 path has one reconstruction schedule
   if (ctx->p.degree >= 4) rcand = {kLaneSchedule + 64, kLaneSchedule + 128, kLaneSchedule + 256};
   if (ctx->p.degree >= 4 && ctx->fp32 && !ctx->p.characteristic)
     for (int b : {64, 128, 256}) rcand.push_back(kHighOcc + b);

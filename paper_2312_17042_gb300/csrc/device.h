@@ -68,6 +68,7 @@ struct DevTables {
   double psibar[kMaxNK];
   double O[kMaxNK][kMaxNK];
   double Phi[kMaxNF][kMaxPerm][kMaxNQ][kMaxNK];
+  double LT[kMaxNK][kMaxNK];                      // see Tables
   double fw[kMaxNQ];
   double vq[kMaxVQ][3];
   double vw[kMaxVQ];
@@ -79,6 +80,9 @@ struct DevTables {
 //   st      int32  [N][M]          stencil ids, directional members first (face after face)
 //   Pc      T      [N][M][nk]      central pseudo-inverse, member-major
 //   Pd      T      [N][NF][PDS]    directional pseudo-inverses (layout of Dir<D, R>)
+//           FP64 path, conserved variables: Pc and Pd hold int2 (h, l), entries of 57-bit integers
+//           (layout in fixed.h)
+//   Pe      int8   [N][kFixExp]    block exponents of those: rows of Pc, then faces of Pd
 //   Uf      T      [N][NF][NQ][NV] face Gauss-point states
 //   nbr     int32  [N][4]          face neighbours, -1 on a boundary
 //   geo     double [N][NF][4]      outward unit normal (n_x, n_y[, n_z]) and area in slot 3;
@@ -96,6 +100,8 @@ struct KArgs {
   const uint32_t *cinfo;
   const void *Pc;
   const void *Pd;
+  const int8_t *Pe;
+  const int2 *phifx;        // FP64 path: the face table (FixShape)
   void *Uf;
   uint8_t *flags;
   const int32_t *nbr;
@@ -125,6 +131,7 @@ struct KArgs {
   float gamma32, gm1_32, eps32, C_T32, inv_lam1_32, one_m_lam1_32, cfl32;
   float fw32[kMaxNQ];
   double fw[kMaxNQ];        // face quadrature weights
+  int8_t phi_exp[kMaxNK];   // block exponents of the face table (FP64 path)
   // gather staging (mixed path): cells in tiles of htile; per tile a record of hrec int32 words
   // [count, 0, 0, 0, distinct member ids ascending, padding]; per cell hms uint16 local indices
   // into its tile's list (stencil members in device order, then the cell itself)
@@ -166,6 +173,7 @@ struct SetupArgs {
   double period[3];
   void *Pc, *Pd;            // outputs, T = double (FP64 path) or float (mixed path)
   int store_fp32;
+  int8_t *Pe;               // not null: Pc, Pd as 57-bit integers, Pe their exponents
   double *geo, *vol;       // vol receives 1 / |V_i|
   float *geo32;
   const DevTables *tab;
@@ -281,8 +289,15 @@ cudaError_t upload_recon_tables_3d(int degree, const Tables &t, cudaStream_t s);
 // gather-staged or streamed schedule on the FP64 path).
 cudaError_t launch_recon_2d(int degree, int fp32, int scheme, const KArgs &a, int block, cudaStream_t s);
 cudaError_t launch_recon_3d(int degree, int fp32, int scheme, const KArgs &a, int block, cudaStream_t s);
+// FP64 path, conserved variables (recon_fixed.cu), at every degree: threads per block.
+cudaError_t launch_recon_fixed(int dim, int degree, int scheme, const KArgs &a, int threads, cudaStream_t s);
 inline cudaError_t launch_recon(int dim, int degree, int fp32, int scheme, const KArgs &a, int block,
                                 cudaStream_t s) {
+  if (!fp32 && !a.characteristic) {  // b and kLaneSchedule + b threads per block
+    const int threads = block >= kLaneSchedule ? block - kLaneSchedule : block;
+    if (threads < 32 || threads > 256 || threads % 32) return cudaErrorInvalidValue;
+    return launch_recon_fixed(dim, degree, scheme, a, threads, s);
+  }
   if (dim == 2 && degree >= 4) return launch_recon_2d_high(degree, fp32, scheme, a, block, s);
   return dim == 2 ? launch_recon_2d(degree, fp32, scheme, a, block, s)
                   : launch_recon_3d(degree, fp32, scheme, a, block, s);

@@ -19,6 +19,7 @@ constexpr int kMaxNQ = 4;    // Gauss points per face (3D; 2D degree 6)
 constexpr int kMaxNV = 5;    // conserved variables in 3D
 constexpr int kMaxDir = 10;  // members of a directional stencil (2d; 10 for the quadratic ones)
 constexpr int kMaxPerm = 6;  // orderings of a face's vertices
+constexpr int kFixExp = 32;  // bytes of a cell's block exponents (FP64 path): K-1 rows, then the faces
 constexpr int kMaxVQ = 16;   // points of the volume rule (4 x 4 in 2D at degree 6)
 
 // K(r,d) of eq. 6: number of monomials of degree <= r in d variables, constant included.
@@ -58,6 +59,12 @@ struct Tables {
   double vq[kMaxVQ][3] = {};            // reference coordinates
   double vw[kMaxVQ] = {};               // weights, sum |V0'| = 1/d!
   int perm_list[kMaxPerm][3] = {};      // permutations of the face's vertex slots
+  // FP64 path: the basis orthonormal in the smoothness form. O = L L^T, b = L^T a, so that
+  // SI = sum b_k^2; LT[k][l] = L_lk (l >= k). Face values of phi' = L^-1 phi as 57-bit integers
+  // h 2^29 + l in units of 2^(phi_exp[k] - 57), where |phi'_k| <= 2^phi_exp[k]
+  double LT[kMaxNK][kMaxNK] = {};
+  int32_t PhiFx[kMaxNF][kMaxPerm][kMaxNQ][kMaxNK][2] = {};
+  int8_t phi_exp[kMaxNK] = {};
 };
 
 void build_tables(int dim, int degree, Tables *t);

@@ -18,6 +18,8 @@ cudaError_t launch_recon_2d_high(int degree, int fp32, int scheme, const KArgs &
 #undef CTENO_OCC
     return cudaSuccess;
   }
+  // FP64: the characteristic reconstruction (conserved variables: recon_fixed.cu)
+  if (!fp32 && !a.characteristic) return cudaErrorInvalidValue;
   if (block < kLaneSchedule + 32 || block > kLaneSchedule + 256 || block % 32) return cudaErrorInvalidValue;
   const int threads = block - kLaneSchedule;
   const int64_t cells_per_block = (int64_t)(threads / 32) * 8;
@@ -31,12 +33,14 @@ cudaError_t launch_recon_2d_high(int degree, int fp32, int scheme, const KArgs &
   if (degree == 5 && fp32 && scheme == 1) CTENO_HIGH(5, float, 1);
   if (degree == 6 && fp32 && scheme == 0) CTENO_HIGH(6, float, 0);
   if (degree == 6 && fp32 && scheme == 1) CTENO_HIGH(6, float, 1);
-  if (degree == 4 && !fp32 && scheme == 0) CTENO_HIGH(4, double, 0);
-  if (degree == 4 && !fp32 && scheme == 1) CTENO_HIGH(4, double, 1);
-  if (degree == 5 && !fp32 && scheme == 0) CTENO_HIGH(5, double, 0);
-  if (degree == 5 && !fp32 && scheme == 1) CTENO_HIGH(5, double, 1);
-  if (degree == 6 && !fp32 && scheme == 0) CTENO_HIGH(6, double, 0);
-  if (degree == 6 && !fp32 && scheme == 1) CTENO_HIGH(6, double, 1);
+#define CTENO_HIGH64(R, SC) launch_stage_kernel(recon_high_kernel<R, double, SC, true>, grid, threads, 0, s, a)
+  if (degree == 4 && !fp32 && scheme == 0) CTENO_HIGH64(4, 0);
+  if (degree == 4 && !fp32 && scheme == 1) CTENO_HIGH64(4, 1);
+  if (degree == 5 && !fp32 && scheme == 0) CTENO_HIGH64(5, 0);
+  if (degree == 5 && !fp32 && scheme == 1) CTENO_HIGH64(5, 1);
+  if (degree == 6 && !fp32 && scheme == 0) CTENO_HIGH64(6, 0);
+  if (degree == 6 && !fp32 && scheme == 1) CTENO_HIGH64(6, 1);
+#undef CTENO_HIGH64
 #undef CTENO_HIGH
   return cudaSuccess;
 }

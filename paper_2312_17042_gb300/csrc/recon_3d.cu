@@ -72,7 +72,8 @@ cudaError_t launch_recon_3d(int degree, int fp32, int scheme, const KArgs &a, in
 #undef CTENO_STAGED
     return cudaSuccess;
   }
-  if (block >= kLaneSchedule) {  // variable-per-lane schedule, block - kLaneSchedule threads
+  if (block >= kLaneSchedule) {  // variable-per-lane schedule, block - kLaneSchedule threads; FP64: the
+                                 // characteristic reconstruction (conserved variables: recon_fixed.cu)
     const int threads = block - kLaneSchedule, cpw = 32 / (3 + 2);
     const int64_t cells_per_block = (int64_t)(threads / 32) * cpw;
     const unsigned grid = (unsigned)((a.N + cells_per_block - 1) / cells_per_block);
@@ -83,25 +84,24 @@ cudaError_t launch_recon_3d(int degree, int fp32, int scheme, const KArgs &a, in
     if (degree == 2 && fp32 && scheme == 1) CTENO_LANES(2, float, 1);
     if (degree == 3 && fp32 && scheme == 0) CTENO_LANES(3, float, 0);
     if (degree == 3 && fp32 && scheme == 1) CTENO_LANES(3, float, 1);
-    if (degree == 2 && !fp32 && scheme == 0) CTENO_LANES(2, double, 0);
-    if (degree == 2 && !fp32 && scheme == 1) CTENO_LANES(2, double, 1);
-    if (degree == 3 && !fp32 && scheme == 0) CTENO_LANES(3, double, 0);
-    if (degree == 3 && !fp32 && scheme == 1) CTENO_LANES(3, double, 1);
+#undef CTENO_LANES
+#define CTENO_LANES(R, SC) launch_stage_kernel(recon_lanes_kernel<3, R, double, SC, true>, grid, threads, 0, s, a)
+    if (degree == 2 && !fp32 && scheme == 0) CTENO_LANES(2, 0);
+    if (degree == 2 && !fp32 && scheme == 1) CTENO_LANES(2, 1);
+    if (degree == 3 && !fp32 && scheme == 0) CTENO_LANES(3, 0);
+    if (degree == 3 && !fp32 && scheme == 1) CTENO_LANES(3, 1);
 #undef CTENO_LANES
     return cudaSuccess;
   }
-  const bool capped = block < 0;  // register-capped variant (FP32 only)
+  if (!fp32) return cudaErrorInvalidValue;  // conserved variables in FP64: recon_fixed.cu
+  const bool capped = block < 0;  // register-capped variant
   if (capped) block = -block;
   const unsigned grid = (unsigned)((a.N + block - 1) / block);
 #define CTENO_RECON(R, T, SC, MB) launch_stage_kernel(recon_kernel<3, R, T, SC, MB>, grid, block, 0, s, a)
-  if (degree == 2 && fp32 && scheme == 0) { if (capped) CTENO_RECON(2, float, 0, 8); else CTENO_RECON(2, float, 0, 0); }
-  if (degree == 2 && fp32 && scheme == 1) { if (capped) CTENO_RECON(2, float, 1, 8); else CTENO_RECON(2, float, 1, 0); }
-  if (degree == 3 && fp32 && scheme == 0) { if (capped) CTENO_RECON(3, float, 0, 8); else CTENO_RECON(3, float, 0, 0); }
-  if (degree == 3 && fp32 && scheme == 1) { if (capped) CTENO_RECON(3, float, 1, 8); else CTENO_RECON(3, float, 1, 0); }
-  if (degree == 2 && !fp32 && scheme == 0) CTENO_RECON(2, double, 0, 0);
-  if (degree == 2 && !fp32 && scheme == 1) CTENO_RECON(2, double, 1, 0);
-  if (degree == 3 && !fp32 && scheme == 0) CTENO_RECON(3, double, 0, 0);
-  if (degree == 3 && !fp32 && scheme == 1) CTENO_RECON(3, double, 1, 0);
+  if (degree == 2 && scheme == 0) { if (capped) CTENO_RECON(2, float, 0, 8); else CTENO_RECON(2, float, 0, 0); }
+  if (degree == 2 && scheme == 1) { if (capped) CTENO_RECON(2, float, 1, 8); else CTENO_RECON(2, float, 1, 0); }
+  if (degree == 3 && scheme == 0) { if (capped) CTENO_RECON(3, float, 0, 8); else CTENO_RECON(3, float, 0, 0); }
+  if (degree == 3 && scheme == 1) { if (capped) CTENO_RECON(3, float, 1, 8); else CTENO_RECON(3, float, 1, 0); }
 #undef CTENO_RECON
   return cudaSuccess;
 }

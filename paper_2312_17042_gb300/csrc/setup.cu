@@ -3,6 +3,7 @@
 // least-squares matrices and the pseudo-inverses P = R^-1 Q^T diag(|V'_m|), so that the
 // coefficients of eq. 12 are a = P (U_m - U_0). One thread per cell; run once per mesh set.
 #include "device.h"
+#include "fixed.h"
 
 namespace cteno {
 namespace {
@@ -103,6 +104,17 @@ __device__ void pinv_column(double (*W)[LD], int rows, int cols, const double *d
     for (int c = k + 1; c < cols; ++c) s -= W[k][c] * out[c];
     out[k] = s / diag[k];
   }
+}
+
+// e with |x| <= 2^e for every |x| <= top, in the range of an int8.
+__device__ __forceinline__ int block_exponent(double top) {
+  return (top > 0.0) ? min(max(ilogb(top) + 1, -100), 100) : 0;
+}
+// x in units of 2^(e - 57) as h 2^29 + l, |l| <= 2^28.
+__device__ __forceinline__ int2 to_fixed(double x, int e) {
+  const long long q = __double2ll_rn(scalbn(x, 57 - e));
+  const long long h = (q + (1 << 28)) >> 29;
+  return make_int2((int)h, (int)(q - h * (1 << 29)));
 }
 
 template <int D, int R>
@@ -251,6 +263,22 @@ __global__ void __launch_bounds__(128) setup_kernel(const SetupArgs a) {
       }
     }
     constexpr int PDS = DR::PDS;
+    if (a.Pe) {  // FP64 path: orthonormal basis, 57-bit integers, member-major
+      double top = 0.0;
+      for (int j = 0; j < ND; ++j)
+        for (int k = 0; k < KD; ++k) {
+          double s = 0.0;
+          for (int l = k; l < KD; ++l) s += T.LT[k][l] * pd[l][j];
+          pd[k][j] = s;
+          top = fmax(top, fabs(s));
+        }
+      const int e = block_exponent(top);
+      a.Pe[i * kFixExp + NK + f] = (int8_t)e;
+      for (int t = 0; t < PDS; ++t)
+        ((int2 *)a.Pd)[(i * NF + f) * PDS + t] = (t < ND * KD) ? to_fixed(pd[t % KD][t / KD], e) : make_int2(0, 0);
+      off += nm;
+      continue;
+    }
     for (int e = 0; e < PDS; ++e) {  // see Dir: member-major (degree <= 3) or unknown-major rows
       const int j = DR::HIGH ? e % DR::NDP : e / KD, k = DR::HIGH ? e / DR::NDP : e % KD;
       const double val = (j < ND && k < KD) ? pd[k][j] : 0.0;
@@ -267,6 +295,30 @@ __global__ void __launch_bounds__(128) setup_kernel(const SetupArgs a) {
   // central stencil
   double dg[NK], vt[NK], bt[NK];
   if (!householder<NK>(W, M, NK, dg, vt, bt)) atomicOr(a.err, kErrRank);
+  if (a.Pe) {  // FP64 path: rows in the orthonormal basis, written as FP64 first, then scaled in place
+    using FX = FixShape<D, R>;
+    double top[NK], *P = (double *)a.Pc;
+    for (int k = 0; k < NK; ++k) top[k] = 0.0;
+    for (int p = 0; p < M; ++p) {
+      double col[NK];
+      pinv_column<NK, M>(W, M, NK, dg, vt, bt, p, col);
+      for (int k = 0; k < NK; ++k) {
+        double s = 0.0;
+        for (int l = k; l < NK; ++l) s += T.LT[k][l] * (col[l] * Vp[p]);
+        P[FX::index(i, p, k)] = s;
+        top[k] = fmax(top[k], fabs(s));
+      }
+    }
+    for (int k = 0; k < NK; ++k) {
+      const int e = block_exponent(top[k]);
+      a.Pe[i * kFixExp + k] = (int8_t)e;
+      for (int p = 0; p < M; ++p) {
+        const int64_t x = FX::index(i, p, k);
+        reinterpret_cast<int2 *>(P)[x] = to_fixed(P[x], e);
+      }
+    }
+    return;
+  }
   for (int p = 0; p < M; ++p) {
     double col[NK];
     pinv_column<NK, M>(W, M, NK, dg, vt, bt, p, col);

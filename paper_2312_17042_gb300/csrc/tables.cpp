@@ -7,8 +7,10 @@
 //
 // Integrals over the reference simplex use the Dirichlet formula
 //   int_{V0'} xi^a eta^b zeta^c = a! b! c! / (a + b + c + d)!.
+#include <algorithm>
 #include <cmath>
 #include <cstring>
+#include <vector>
 
 #include "internal.h"
 
@@ -19,6 +21,21 @@ double fact(int n) {
   double f = 1.0;
   for (int i = 2; i <= n; ++i) f *= i;
   return f;
+}
+
+// An unevaluated sum of two doubles (about 106 bits), and s + a x in it (error-free transformations:
+// Knuth's two-sum, the product's error by a fused multiply-add).
+struct Double2 {
+  double hi = 0.0, lo = 0.0;
+};
+Double2 two_sum(double a, double b) {
+  const double s = a + b, t = s - a;
+  return {s, (a - (s - t)) + (b - t)};
+}
+Double2 add_product(const Double2 &s, double a, const Double2 &x) {
+  const double p = a * x.hi, e = std::fma(a, x.hi, -p) + a * x.lo;
+  const Double2 r = two_sum(s.hi, p);
+  return two_sum(r.hi, r.lo + (s.lo + e));
 }
 
 // int over V0' of xi^e (e[0..d-1]).
@@ -276,6 +293,46 @@ void build_tables(int dim, int degree, Tables *t) {
         for (int i = 0; i < k; ++i)
           t->Phi[f][p][q][i] = eval_monomial(t->ex[i], xi, d) - t->psibar[i];
       }
+  }
+  // the orthonormal basis: L from O, then phi' = L^-1 phi at the face points of this very L in
+  // double-double arithmetic (b^T phi' = a^T phi whatever L's own rounding)
+  double L[kMaxNK][kMaxNK] = {};
+  for (int j = 0; j < k; ++j)
+    for (int i = j; i < k; ++i) {
+      double s = t->O[i][j];
+      for (int l = 0; l < j; ++l) s -= L[i][l] * L[j][l];
+      L[i][j] = (i == j) ? std::sqrt(s) : s / L[j][j];
+      t->LT[j][i] = L[i][j];
+    }
+  std::vector<Double2> y((size_t)kMaxNF * kMaxPerm * kMaxNQ * kMaxNK);
+  auto at = [&](int f, int p, int q) { return &y[(size_t)((f * kMaxPerm + p) * kMaxNQ + q) * kMaxNK]; };
+  double top[kMaxNK] = {};
+  for (int f = 0; f < t->nf; ++f)
+    for (int p = 0; p < t->nperm; ++p)
+      for (int q = 0; q < t->nq; ++q) {
+        Double2 *v = at(f, p, q);
+        for (int i = 0; i < k; ++i) {
+          Double2 s{t->Phi[f][p][q][i], 0.0};
+          for (int l = 0; l < i; ++l) s = add_product(s, -L[i][l], v[l]);
+          const double hi = s.hi / L[i][i];
+          const Double2 r = add_product(s, -L[i][i], Double2{hi, 0.0});
+          v[i] = two_sum(hi, (r.hi + r.lo) / L[i][i]);
+          top[i] = std::max(top[i], std::fabs(v[i].hi));
+        }
+      }
+  for (int i = 0; i < k; ++i) {
+    int e = 0;
+    std::frexp(top[i], &e);  // |phi'_i| < 2^e
+    t->phi_exp[i] = (int8_t)e;
+    for (int f = 0; f < t->nf; ++f)
+      for (int p = 0; p < t->nperm; ++p)
+        for (int q = 0; q < t->nq; ++q) {
+          const Double2 v = at(f, p, q)[i];
+          const int64_t x = std::llrint(std::ldexp(v.hi, 57 - e)) + std::llrint(std::ldexp(v.lo, 57 - e));
+          const int64_t h = (x + (1 << 28)) >> 29;
+          t->PhiFx[f][p][q][i][0] = (int32_t)h;
+          t->PhiFx[f][p][q][i][1] = (int32_t)(x - h * (1 << 29));
+        }
   }
 }
 
