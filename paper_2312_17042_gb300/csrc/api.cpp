@@ -315,6 +315,7 @@ int cteno_create(cteno_ctx **out, const cteno_params *p, void *cuda_stream) {
   ctx->nd = dir_members(p->dim, p->degree);
   // the variable-per-lane schedule for degrees 4 to 6 and for the characteristic reconstruction
   if (p->degree >= 4 || p->characteristic) ctx->recon_block = kLaneSchedule + 128;
+  if (p->precision == CTENO_FP64) ctx->flux_block = 32;  // see flux64.cuh
   ctx->nsel = p->characteristic ? ctx->nf * ctx->nv : ctx->nv;
   ctx->nst = p->rk;
   ctx->fp32 = (p->precision == CTENO_MIXED);
@@ -1115,6 +1116,7 @@ int cteno_autotune(cteno_ctx *ctx, int32_t *best_out) {
   }
   std::vector<int> fcand = cand;  // flux: also the face-based schedule
   for (int b : {kFaceFlux + 128, kFaceFlux + 256}) fcand.push_back(b);
+  if (!ctx->fp32) fcand = {32, 64, 128};  // the FP64 path has one flux schedule
   for (int b : fcand) {
     float tot = 0;
     for (int r = 0; r < reps; ++r) {

@@ -12,35 +12,20 @@
 namespace cteno {
 namespace {
 
-// Reciprocal, quotient and square root: IEEE operations on the FP64 path; on the mixed path the
-// GPU's single-instruction approximations (relative error about 2^-23, subnormal operands flushed
-// to zero: densities, pressures and wave-speed differences of physical states are normal numbers).
-// Both cells of a face run the same instruction sequence on the same operands, so their face
-// values stay bit-identical.
-template <typename T>
-__device__ __forceinline__ T rcp_(T x) {
-  if constexpr (sizeof(T) == 4) {
-    float y;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return y;
-  } else {
-    return 1.0 / x;
-  }
+// Reciprocal, quotient and square root of the mixed path: the GPU's single-instruction
+// approximations (relative error about 2^-23, subnormal operands flushed to zero: densities, pressures
+// and wave-speed differences of physical states are normal numbers). Both cells of a face run the same
+// instruction sequence on the same operands, so their face values stay bit-identical.
+__device__ __forceinline__ float rcp_(float x) {
+  float y;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
 }
-template <typename T>
-__device__ __forceinline__ T div_(T x, T y) {
-  if constexpr (sizeof(T) == 4) return x * rcp_<T>(y);
-  else return x / y;
-}
-template <typename T>
-__device__ __forceinline__ T sqrt_(T x) {
-  if constexpr (sizeof(T) == 4) {
-    float y;
-    asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return y;
-  } else {
-    return sqrt(x);
-  }
+__device__ __forceinline__ float div_(float x, float y) { return x * rcp_(y); }
+__device__ __forceinline__ float sqrt_(float x) {
+  float y;
+  asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
 }
 
 // Finite FP64 value (exponent field not all ones), tested with integer operations.
@@ -94,8 +79,8 @@ __device__ __forceinline__ void wall_mirror(const T *u, const T *n, T *o) {
   o[D + 1] = u[D + 1];
 }
 
-template <int D, typename T>
-__device__ __forceinline__ void physical_flux(const T *u, const T *n, T p, T un, T *F) {
+template <int D>
+__device__ __forceinline__ void physical_flux(const float *u, const float *n, float p, float un, float *F) {
   F[0] = u[0] * un;
 #pragma unroll
   for (int j = 0; j < D; ++j) F[1 + j] = u[1 + j] * un + p * n[j];
@@ -105,12 +90,12 @@ __device__ __forceinline__ void physical_flux(const T *u, const T *n, T p, T un,
 // HLLC flux through a face with unit normal n from state uL (inside) to uR (outside). Wave
 // speeds of eq. 25 with the Roe averages of eq. 26 (full averaged velocity in the sound speed),
 // contact speed and star pressure of eq. 28, star states of eq. 29 in vector form.
-template <int D, typename T>
-__device__ __forceinline__ void hllc(const T *uL, const T *uR, const T *n, T g, T *F) {
+template <int D>
+__device__ __forceinline__ void hllc(const float *uL, const float *uR, const float *n, float g, float *F) {
   constexpr int NV = D + 2;
-  const T rL = uL[0], rR = uR[0];
-  const T iL = rcp_<T>(rL), iR = rcp_<T>(rR);
-  T vL[D], vR[D], unL = 0, unR = 0, kL = 0, kR = 0;
+  const float rL = uL[0], rR = uR[0];
+  const float iL = rcp_(rL), iR = rcp_(rR);
+  float vL[D], vR[D], unL = 0, unR = 0, kL = 0, kR = 0;
 #pragma unroll
   for (int j = 0; j < D; ++j) {
     vL[j] = uL[1 + j] * iL;
@@ -120,39 +105,39 @@ __device__ __forceinline__ void hllc(const T *uL, const T *uR, const T *n, T g, 
     kL += vL[j] * uL[1 + j];
     kR += vR[j] * uR[1 + j];
   }
-  const T pL = (g - (T)1) * (uL[NV - 1] - (T)0.5 * kL);
-  const T pR = (g - (T)1) * (uR[NV - 1] - (T)0.5 * kR);
-  const T cL = sqrt_<T>(g * pL * iL), cR = sqrt_<T>(g * pR * iR);
-  const T HL = (uL[NV - 1] + pL) * iL, HR = (uR[NV - 1] + pR) * iR;
-  const T Dr = sqrt_<T>(rR * iL);
-  const T idn = rcp_<T>((T)1 + Dr);
-  T ut2 = 0, utn = 0;
+  const float pL = (g - (float)1) * (uL[NV - 1] - (float)0.5 * kL);
+  const float pR = (g - (float)1) * (uR[NV - 1] - (float)0.5 * kR);
+  const float cL = sqrt_(g * pL * iL), cR = sqrt_(g * pR * iR);
+  const float HL = (uL[NV - 1] + pL) * iL, HR = (uR[NV - 1] + pR) * iR;
+  const float Dr = sqrt_(rR * iL);
+  const float idn = rcp_((float)1 + Dr);
+  float ut2 = 0, utn = 0;
 #pragma unroll
   for (int j = 0; j < D; ++j) {
-    const T ut = (vL[j] + vR[j] * Dr) * idn;
+    const float ut = (vL[j] + vR[j] * Dr) * idn;
     ut2 += ut * ut;
     utn += ut * n[j];
   }
-  const T Ht = (HL + HR * Dr) * idn;
-  const T ct = sqrt_<T>((g - (T)1) * (Ht - (T)0.5 * ut2));
-  const T SL = fmin(unL - cL, utn - ct);
-  const T SR = fmax(unR + cR, utn + ct);
-  const T SM = div_<T>(rR * unR * (SR - unR) - rL * unL * (SL - unL) + pL - pR,
+  const float Ht = (HL + HR * Dr) * idn;
+  const float ct = sqrt_((g - (float)1) * (Ht - (float)0.5 * ut2));
+  const float SL = fmin(unL - cL, utn - ct);
+  const float SR = fmax(unR + cR, utn + ct);
+  const float SM = div_(rR * unR * (SR - unR) - rL * unL * (SL - unL) + pL - pR,
                        rR * (SR - unR) - rL * (SL - unL));
   // The four cases, tested in the order SL > 0 (left state), SM > 0 (left star state), SR > 0
   // (right star state), else (right state), evaluated without branches (neighbouring faces of a
   // warp take different cases): the operands of side k are selected, the star correction is
   // dropped in the two supersonic cases. Each case's arithmetic is the same as written out alone.
-  const bool left = (SL > (T)0) || (SM > (T)0);
-  const bool sup = (SL > (T)0) || (!(SM > (T)0) && !(SR > (T)0));
-  T uk[NV];
+  const bool left = (SL > (float)0) || (SM > (float)0);
+  const bool sup = (SL > (float)0) || (!(SM > (float)0) && !(SR > (float)0));
+  float uk[NV];
 #pragma unroll
   for (int v = 0; v < NV; ++v) uk[v] = left ? uL[v] : uR[v];
-  const T pk = left ? pL : pR, unk = left ? unL : unR, Sk = left ? SL : SR, rk = uk[0];
-  physical_flux<D, T>(uk, n, pk, unk, F);
-  const T ps = rL * (unL - SL) * (unL - SM) + pL;
-  const T fct = rcp_<T>(Sk - SM), a = Sk - unk;
-  T G[NV];
+  const float pk = left ? pL : pR, unk = left ? unL : unR, Sk = left ? SL : SR, rk = uk[0];
+  physical_flux<D>(uk, n, pk, unk, F);
+  const float ps = rL * (unL - SL) * (unL - SM) + pL;
+  const float fct = rcp_(Sk - SM), a = Sk - unk;
+  float G[NV];
   G[0] = F[0] + Sk * (rk * a * fct - uk[0]);
 #pragma unroll
   for (int j = 0; j < D; ++j) G[1 + j] = F[1 + j] + Sk * ((a * uk[1 + j] + (ps - pk) * n[j]) * fct - uk[1 + j]);
@@ -227,36 +212,32 @@ __device__ __forceinline__ void warp_min_to(double *dt, int slot, double v) {
   }
 }
 
-// Local CFL step of one cell: |V_i| / sum_f |A_f| (|u_i . n_f| + c_i), in the path's arithmetic
-// type (FP64 geometry for the FP64 path; FP32 values and geometry for the mixed path, where the
-// step only sets the time-step size).
-template <int D, typename T>
-__device__ __forceinline__ double local_dt(const KArgs &a, int64_t i, const T *uu) {
+// Local CFL step of one cell of the mixed path, |V_i| / sum_f |A_f| (|u_i . n_f| + c_i), in FP32 values
+// and geometry (the step only sets the time-step size).
+template <int D>
+__device__ __forceinline__ double local_dt(const KArgs &a, int64_t i, const float *uu) {
   constexpr int NF = D + 1;
-  constexpr bool F32 = sizeof(T) == 4;
-  const T *G = F32 ? (const T *)a.geo32 : (const T *)a.geo;
-  T g;
-  if constexpr (F32) g = a.gamma32; else g = a.gamma;
-  const T ir = rcp_<T>(uu[0]);
-  T ke = 0, u[D];
+  const float *G = a.geo32;
+  const float g = a.gamma32;
+  const float ir = rcp_(uu[0]);
+  float ke = 0, u[D];
 #pragma unroll
   for (int j = 0; j < D; ++j) {
     u[j] = uu[1 + j] * ir;
     ke += uu[1 + j] * u[j];
   }
-  const T p = (g - (T)1) * (uu[D + 1] - (T)0.5 * ke);
-  const T c = sqrt_<T>(g * p * ir);
-  T s = 0;
+  const float p = (g - 1.0f) * (uu[D + 1] - 0.5f * ke);
+  const float c = sqrt_(g * p * ir);
+  float s = 0;
 #pragma unroll
   for (int f = 0; f < NF; ++f) {
-    const T *gf = G + (i * NF + f) * 4;
-    T un = 0;
+    const float *gf = G + (i * NF + f) * 4;
+    float un = 0;
 #pragma unroll
     for (int j = 0; j < D; ++j) un += u[j] * gf[j];
     s += gf[3] * (fabs(un) + c);
   }
-  if constexpr (F32) return (double)rcp_<float>(s * (float)a.vol[i]);
-  else return 1.0 / (s * a.vol[i]);
+  return (double)rcp_(s * (float)a.vol[i]);
 }
 
 // Error-free sum of two FP32 values (Knuth's TwoSum): s + e == a + b exactly.
@@ -273,12 +254,11 @@ __device__ __forceinline__ void two_sum(float a, float b, float &s, float &e) {
 // U^{n+1} = 1/3 U^n + 2/3 (U2 + dt R(U2)); or the classical RK4 with its running sum in Acc:
 // Acc = U^n + dt/6 k1, U = U^n + dt/2 k1; Acc += dt/3 k2, U = U^n + dt/2 k2; Acc += dt/3 k3,
 // U = U^n + dt k3; U^{n+1} = Acc + dt/6 k4.
-template <int D, typename T>
+template <int D>
 __device__ __forceinline__ void stage_tail(const KArgs &a, const int64_t i, const bool active,
                                            const double (&u64)[Lay<D>::NVP], const double (&acc)[Lay<D>::NV]) {
   using L = Lay<D>;
   constexpr int NV = L::NV, NVP = L::NVP;
-  constexpr bool F32 = sizeof(T) == 4;
   const int mesh = (a.nmesh > 1) ? mesh_of(a, i) : 0;
   const double dtv = a.dt[mesh] * a.vol[i];  // dt / |V_i|
   double un[NVP], res[NVP], ac[NVP];
@@ -338,34 +318,29 @@ __device__ __forceinline__ void stage_tail(const KArgs &a, const int64_t i, cons
         reinterpret_cast<double2 *>(a.Acc + i * NVP)[c] = make_double2(ac[2 * c], ac[2 * c + 1]);
     }
   }
-  T ust[NVP];  // the new state in the path's type, for the CFL step
-  if constexpr (F32) {  // FP32 (hi, lo) shadow of the new state
-    float4 hl[NVP / 2];
+  float ust[NVP];  // the FP32 (hi, lo) shadow of the new state; hi also for the CFL step
+  float4 hl[NVP / 2];
 #pragma unroll
-    for (int c = 0; c < NVP / 2; ++c) {
-      const float2 s0 = f64_split(res[2 * c]), s1 = f64_split(res[2 * c + 1]);
-      hl[c] = make_float4(s0.x, s0.y, s1.x, s1.y);
-      ust[2 * c] = s0.x;
-      ust[2 * c + 1] = s1.x;
-    }
-    if (active) {
+  for (int c = 0; c < NVP / 2; ++c) {
+    const float2 s0 = f64_split(res[2 * c]), s1 = f64_split(res[2 * c + 1]);
+    hl[c] = make_float4(s0.x, s0.y, s1.x, s1.y);
+    ust[2 * c] = s0.x;
+    ust[2 * c + 1] = s1.x;
+  }
+  if (active) {
 #pragma unroll
-      for (int c = 0; c < NVP / 2; ++c) reinterpret_cast<float4 *>(a.U32 + i * 2 * NVP)[c] = hl[c];
-    }
-  } else {
-#pragma unroll
-    for (int v = 0; v < NVP; ++v) ust[v] = res[v];
+    for (int c = 0; c < NVP / 2; ++c) reinterpret_cast<float4 *>(a.U32 + i * 2 * NVP)[c] = hl[c];
   }
   if (!finite && active) atomicOr(a.err, kErrNonFinite);
   if (a.stage == a.last_stage)
-    warp_min_to(a.dt, a.nmesh + mesh, (finite && active) ? a.cfl * local_dt<D, T>(a, i, ust) : 1e300);
+    warp_min_to(a.dt, a.nmesh + mesh, (finite && active) ? a.cfl * local_dt<D>(a, i, ust) : 1e300);
 }
 
-template <int D, typename T, int MINB, int NQ>
+template <int D, int MINB, int NQ>
 __global__ void __launch_bounds__(MINB ? 128 : 256, MINB ? MINB : 1) flux_kernel(const KArgs a) {
   using L = Lay<D>;
   constexpr int NV = L::NV, NVP = L::NVP, NF = L::NF, FB = NQ * NV;
-  constexpr bool F32 = sizeof(T) == 4;
+  using T = float;
   pdl_wait(a);  // face states of the reconstruction, the state of the previous stage
   const int64_t N = a.N;
   const int64_t cell = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -374,9 +349,8 @@ __global__ void __launch_bounds__(MINB ? 128 : 256, MINB ? MINB : 1) flux_kernel
   const bool active = cell < N;
   const int64_t i = active ? cell : N - 1;
   const T *__restrict__ Uf = (const T *)a.Uf;
-  const T *__restrict__ G = F32 ? (const T *)a.geo32 : (const T *)a.geo;
-  T g;
-  if constexpr (F32) g = a.gamma32; else g = a.gamma;
+  const T *__restrict__ G = a.geo32;
+  const T g = a.gamma32;
   const uint32_t meta = __ldg(a.fmeta + i);
   const int4 nb4 = __ldg(reinterpret_cast<const int4 *>(a.nbr) + i);
   const int nbv[4] = {nb4.x, nb4.y, nb4.z, nb4.w};
@@ -392,7 +366,6 @@ __global__ void __launch_bounds__(MINB ? 128 : 256, MINB ? MINB : 1) flux_kernel
   float acc_hi[NV], acc_lo[NV];
 #pragma unroll
   for (int v = 0; v < NV; ++v) {
-    acc[v] = 0.0;
     acc_hi[v] = 0.0f;
     acc_lo[v] = 0.0f;
   }
@@ -429,10 +402,9 @@ __global__ void __launch_bounds__(MINB ? 128 : 256, MINB ? MINB : 1) flux_kernel
 #pragma unroll
       for (int q = 0; q < NQ; ++q) {
         T F[NV];
-        if (own) hllc<D, T>(uI[ff] + q * NV, uO[ff] + q * NV, n, g, F);
-        else hllc<D, T>(uO[ff] + q * NV, uI[ff] + q * NV, n, g, F);
-        T w;
-    if constexpr (F32) w = a.fw32[q]; else w = a.fw[q];
+        if (own) hllc<D>(uI[ff] + q * NV, uO[ff] + q * NV, n, g, F);
+        else hllc<D>(uO[ff] + q * NV, uI[ff] + q * NV, n, g, F);
+        const T w = a.fw32[q];
 #pragma unroll
         for (int v = 0; v < NV; ++v) Ff[v] = (q == 0) ? w * F[v] : Ff[v] + w * F[v];
       }
@@ -440,34 +412,28 @@ __global__ void __launch_bounds__(MINB ? 128 : 256, MINB ? MINB : 1) flux_kernel
       for (int v = 0; v < NV; ++v) {
         const T x = gf[ff][3] * Ff[v];
         const T c = own ? x : -x;  // the exact negative of the other cell's value
-        if constexpr (F32) {
-          // exact FP32 accumulation over the faces: running (hi, lo) by TwoSum
-          float s, e;
-          two_sum(acc_hi[v], c, s, e);
-          acc_hi[v] = s;
-          acc_lo[v] += e;
-        } else {
-          acc[v] += c;  // FP64 accumulation over the faces
-        }
+        // exact FP32 accumulation over the faces: running (hi, lo) by TwoSum
+        float s, e;
+        two_sum(acc_hi[v], c, s, e);
+        acc_hi[v] = s;
+        acc_lo[v] += e;
       }
     }
   }
-  if constexpr (F32) {
 #pragma unroll
-    for (int v = 0; v < NV; ++v) acc[v] = f32_to_f64(acc_hi[v]) + f32_to_f64(acc_lo[v]);
-  }
-  stage_tail<D, T>(a, i, active, u64, acc);
+  for (int v = 0; v < NV; ++v) acc[v] = f32_to_f64(acc_hi[v]) + f32_to_f64(acc_lo[v]);
+  stage_tail<D>(a, i, active, u64, acc);
 }
 
 // Face flux of the face-based schedule: one thread per face, HLLC at the face's Gauss points in
 // its owner's orientation (the same operands and order as flux_kernel's owner side), weighted and
 // scaled by the area; record e holds |A| sum_q w_q F_q, padded to NFP values.
-template <int D, typename T, int NQ>
+template <int D, int NQ>
 __global__ void __launch_bounds__(256) face_flux_kernel(const KArgs a) {
   using L = Lay<D>;
   constexpr int NV = L::NV, NVP = L::NVP, NF = L::NF, FB = NQ * NV;
   constexpr int NFP = (NV + 3) & ~3;
-  constexpr bool F32 = sizeof(T) == 4;
+  using T = float;
   pdl_wait(a);  // face states of the reconstruction
   const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= a.nfaces) return;
@@ -475,9 +441,8 @@ __global__ void __launch_bounds__(256) face_flux_kernel(const KArgs a) {
   const int64_t i = codes.x >> 2;
   const int f = codes.x & 3;
   const T *__restrict__ Uf = (const T *)a.Uf;
-  const T *__restrict__ G = F32 ? (const T *)a.geo32 : (const T *)a.geo;
-  T g;
-  if constexpr (F32) g = a.gamma32; else g = a.gamma;
+  const T *__restrict__ G = a.geo32;
+  const T g = a.gamma32;
   T gf[4], uI[FB], uO[FB];
   load16<T, 4>(G + (i * NF + f) * 4, gf);
   load16<T, FB>(Uf + (i * NF + f) * FB, uI);
@@ -498,9 +463,8 @@ __global__ void __launch_bounds__(256) face_flux_kernel(const KArgs a) {
 #pragma unroll
   for (int q = 0; q < NQ; ++q) {
     T F[NV];
-    hllc<D, T>(uI + q * NV, uO + q * NV, n, g, F);
-    T w;
-    if constexpr (F32) w = a.fw32[q]; else w = a.fw[q];
+    hllc<D>(uI + q * NV, uO + q * NV, n, g, F);
+    const T w = a.fw32[q];
 #pragma unroll
     for (int v = 0; v < NV; ++v) Ff[v] = (q == 0) ? w * F[v] : Ff[v] + w * F[v];
   }
@@ -512,11 +476,11 @@ __global__ void __launch_bounds__(256) face_flux_kernel(const KArgs a) {
 
 // Residual and stage update of the face-based schedule: as flux_kernel with its face fluxes read
 // from face_flux_kernel's records.
-template <int D, typename T, int MINB>
-__global__ void __launch_bounds__(MINB ? 128 : 256, MINB ? MINB : 1) cell_update_kernel(const KArgs a) {
+template <int D>
+__global__ void __launch_bounds__(256) cell_update_kernel(const KArgs a) {
   using L = Lay<D>;
   constexpr int NV = L::NV, NVP = L::NVP, NF = L::NF;
-  constexpr bool F32 = sizeof(T) == 4;
+  using T = float;
   pdl_wait(a);  // the face fluxes of this stage
   const int64_t N = a.N;
   const int64_t cell = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -536,7 +500,6 @@ __global__ void __launch_bounds__(MINB ? 128 : 256, MINB ? MINB : 1) cell_update
   float acc_hi[NV], acc_lo[NV];
 #pragma unroll
   for (int v = 0; v < NV; ++v) {
-    acc[v] = 0.0;
     acc_hi[v] = 0.0f;
     acc_lo[v] = 0.0f;
   }
@@ -554,26 +517,21 @@ __global__ void __launch_bounds__(MINB ? 128 : 256, MINB ? MINB : 1) cell_update
 #pragma unroll
     for (int v = 0; v < NV; ++v) {
       const T c = neg ? -x[v] : x[v];
-      if constexpr (F32) {
-        float s, er;
-        two_sum(acc_hi[v], c, s, er);
-        acc_hi[v] = s;
-        acc_lo[v] += er;
-      } else {
-        acc[v] += c;
-      }
+      float s, er;
+      two_sum(acc_hi[v], c, s, er);
+      acc_hi[v] = s;
+      acc_lo[v] += er;
     }
   }
-  if constexpr (F32) {
 #pragma unroll
-    for (int v = 0; v < NV; ++v) acc[v] = f32_to_f64(acc_hi[v]) + f32_to_f64(acc_lo[v]);
-  }
-  stage_tail<D, T>(a, i, active, u64, acc);
+  for (int v = 0; v < NV; ++v) acc[v] = f32_to_f64(acc_hi[v]) + f32_to_f64(acc_lo[v]);
+  stage_tail<D>(a, i, active, u64, acc);
 }
 
 }  // namespace
 }  // namespace cteno
 
+#include "flux64.cuh"
 #include "flux_lanes.cuh"
 
 namespace cteno {
@@ -596,7 +554,10 @@ __global__ void dt_kernel(const KArgs a, int64_t first, int64_t count) {
     else uu[v] = u[v];
   }
   const int mesh = (a.nmesh > 1) ? mesh_of(a, i) : 0;
-  warp_min_to(a.dt, a.nmesh + mesh, active ? a.cfl * local_dt<D, T>(a, i, uu) : 1e300);
+  double dt;
+  if constexpr (sizeof(T) == 4) dt = a.cfl * local_dt<D>(a, i, uu);
+  else dt = a.cfl * local_dt64<D>(a, i, uu);
+  warp_min_to(a.dt, a.nmesh + mesh, active ? dt : 1e300);
 }
 
 __global__ void time_advance_kernel(double *time, const double *dt, int nmesh) {
@@ -651,7 +612,10 @@ __global__ void permute_in_all_dt_kernel(const KArgs a, const int32_t *grank, co
       }
     }
   }
-  warp_min_to(a.dt, a.nmesh + k, active ? a.cfl * local_dt<D, T>(a, g, ut) : 1e300);
+  double dt;
+  if constexpr (sizeof(T) == 4) dt = a.cfl * local_dt<D>(a, g, ut);
+  else dt = a.cfl * local_dt64<D>(a, g, ut);
+  warp_min_to(a.dt, a.nmesh + k, active ? dt : 1e300);
 }
 
 __global__ void permute_out_all_kernel(int nv, int nvp, int64_t N, int nmesh, const int64_t *mesh_off,
@@ -697,35 +661,31 @@ namespace {
 // The flux kernels of dimension D with NQ Gauss points per face.
 template <int D, int NQ>
 void launch_flux_nq(int fp32, const KArgs &a, int block, cudaStream_t s) {
+  if (!fp32) {  // one schedule (flux64.cuh); b, kLaneSchedule + b, kFaceFlux + b threads per block
+    const int threads = block >= kFaceFlux ? block - kFaceFlux : block >= kLaneSchedule ? block - kLaneSchedule : block;
+    const int warps = threads / 32;
+    launch_stage_kernel(face_flux64_kernel<D, NQ>, grid_for(a.nfaces, warps * (32 / NQ)), threads, 0, s, a);
+    launch_stage_kernel(cell_update64_kernel<D>, grid_for(a.N, warps * (32 / (D + 2))), threads, 0, s, a);
+    return;
+  }
   if (block >= kFaceFlux) {  // face-based: HLLC once per face, then the per-cell gather and update
     const int threads = block - kFaceFlux;
-    const unsigned gf = grid_for(a.nfaces, 256), gc = grid_for(a.N, threads);
-    if (fp32) {
-      launch_stage_kernel(face_flux_kernel<D, float, NQ>, gf, 256, 0, s, a);
-      launch_stage_kernel(cell_update_kernel<D, float, 0>, gc, threads, 0, s, a);
-    } else {
-      launch_stage_kernel(face_flux_kernel<D, double, NQ>, gf, 256, 0, s, a);
-      launch_stage_kernel(cell_update_kernel<D, double, 0>, gc, threads, 0, s, a);
-    }
+    launch_stage_kernel(face_flux_kernel<D, NQ>, grid_for(a.nfaces, 256), 256, 0, s, a);
+    launch_stage_kernel(cell_update_kernel<D>, grid_for(a.N, threads), threads, 0, s, a);
     return;
   }
   if (block >= kLaneSchedule) {  // face-per-lane schedule, block - kLaneSchedule threads
     const int threads = block - kLaneSchedule, cpw = 32 / (D + 1);
     const int64_t cells_per_block = (int64_t)(threads / 32) * cpw;
     const unsigned grid = (unsigned)((a.N + cells_per_block - 1) / cells_per_block);
-    if (fp32) launch_stage_kernel(flux_lanes_kernel<D, float, NQ>, grid, threads, 0, s, a);
-    else launch_stage_kernel(flux_lanes_kernel<D, double, NQ>, grid, threads, 0, s, a);
+    launch_stage_kernel(flux_lanes_kernel<D, NQ>, grid, threads, 0, s, a);
     return;
   }
-  const bool capped = block < 0;  // register-capped variant (FP32 only)
+  const bool capped = block < 0;  // register-capped variant
   if (capped) block = -block;
   const unsigned grid = grid_for(a.N, block);
-  if (fp32) {
-    if (capped) launch_stage_kernel(flux_kernel<D, float, 8, NQ>, grid, block, 0, s, a);
-    else launch_stage_kernel(flux_kernel<D, float, 0, NQ>, grid, block, 0, s, a);
-  } else {
-    launch_stage_kernel(flux_kernel<D, double, 0, NQ>, grid, block, 0, s, a);
-  }
+  if (capped) launch_stage_kernel(flux_kernel<D, 8, NQ>, grid, block, 0, s, a);
+  else launch_stage_kernel(flux_kernel<D, 0, NQ>, grid, block, 0, s, a);
 }
 }  // namespace
 

@@ -1,0 +1,257 @@
+// flux64.cuh -- the flux and stage update of the FP64 path (included by flux.cu after boundary_state,
+// the time-step reduction and TwoSum helpers).
+//
+// Both kernels are bound by the FP64 pipe, which takes a warp instruction every 64 clocks per
+// scheduler whatever its other load, so they spend as few FP64 instructions as they can and spread
+// them over as many warps as the mesh gives:
+//   face_flux64    one lane per face Gauss point (not per face): HLLC once per face in its owner's
+//                  orientation, comparisons and selections on integers, reciprocals and square roots
+//                  from the FP32-accurate hardware estimate and a third-order (Halley) or two
+//                  Newton-type corrections; the points of a face are summed by shuffles;
+//   cell_update64  one lane per conserved variable: the cell's face fluxes, signed, in face order,
+//                  the Runge-Kutta update and, over the same lanes, the CFL step.
+// The per-cell schedules of the mixed path evaluate every face twice; in FP64 they took three times
+// as long and are not built.
+//
+// Measured, both kernels, against the per-cell schedule (the default then) and the face-based one with
+// a lane per face: 131 072 triangles, 2 points an edge 499 / 165 -> 121 us; 24 576 tetrahedra 362 / 122
+// -> 74 us; 4200 triangles, 3 points 123 / 49 -> 15 us; 2048 triangles 80 / 33 -> 13 us. The large
+// ones run at 80 % of the FP64 pipe. Small meshes want many small blocks (4200 triangles: 15.2 us in blocks
+// of 32 threads, 18.3 in blocks of 128), large ones do not care (121.7 / 121.2 us): 32 by default.
+#pragma once
+
+namespace cteno {
+namespace {
+
+// 1 / x to about one unit in the last place: y (1 + e + e^2), e = 1 - x y, from an estimate y with
+// |e| < 2^-19. Normal x.
+__device__ __forceinline__ double rcp64(const double x) {
+  double y;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  const double e = fma(-x, y, 1.0);
+  return fma(y, fma(e, e, e), y);
+}
+// sqrt(x): coupled iteration on g ~ sqrt(x) and h ~ 1 / (2 sqrt(x)) (Goldschmidt), then the
+// residual correction g + (x - g^2) h. Values below the normal numbers give 0.
+__device__ __forceinline__ double sqrt64(const double x) {
+  double y;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  double g = x * y, h = __hiloint2double(__double2hiint(y) - (1 << 20), __double2loint(y));  // y / 2
+  const double r = fma(-g, h, 0.5);
+  g = fma(g, r, g);
+  h = fma(h, r, h);
+  g = fma(fma(-g, g, x), h, g);
+  return (__double2hiint(x) & 0x7FFFFFFF) < 0x00100000 ? 0.0 : g;
+}
+// x > 0, a < b, on integers.
+__device__ __forceinline__ bool positive64(const double x) {
+  const int h = __double2hiint(x);
+  return (h > 0 && h <= 0x7FF00000) || (h == 0 && __double2loint(x) != 0);
+}
+__device__ __forceinline__ bool less64(const double a, const double b) {
+  const long long x = __double_as_longlong(a), y = __double_as_longlong(b);
+  return (x ^ ((x >> 63) & 0x7FFFFFFFFFFFFFFFll)) < (y ^ ((y >> 63) & 0x7FFFFFFFFFFFFFFFll));
+}
+
+// HLLC flux as hllc() (eqs. 24-29), with common factors taken once: about 125 FP64 instructions in 2D
+// and 140 in 3D, against 187 with IEEE division and square root.
+template <int D>
+__device__ __forceinline__ void hllc64(const double *uL, const double *uR, const double *n, const double g, double *F) {
+  constexpr int NV = D + 2;
+  const double rL = uL[0], rR = uR[0], gm1 = g - 1.0;
+  const double iL = rcp64(rL), iR = rcp64(rR);
+  double vL[D], vR[D], unL, unR, kL, kR;
+#pragma unroll
+  for (int j = 0; j < D; ++j) {
+    vL[j] = uL[1 + j] * iL;
+    vR[j] = uR[1 + j] * iR;
+    unL = j ? fma(vL[j], n[j], unL) : vL[j] * n[j];
+    unR = j ? fma(vR[j], n[j], unR) : vR[j] * n[j];
+    kL = j ? fma(vL[j], uL[1 + j], kL) : vL[j] * uL[1 + j];
+    kR = j ? fma(vR[j], uR[1 + j], kR) : vR[j] * uR[1 + j];
+  }
+  const double pL = gm1 * fma(-0.5, kL, uL[NV - 1]), pR = gm1 * fma(-0.5, kR, uR[NV - 1]);
+  const double cL = sqrt64(g * pL * iL), cR = sqrt64(g * pR * iR);
+  const double HL = (uL[NV - 1] + pL) * iL, HR = (uR[NV - 1] + pR) * iR;
+  const double Dr = sqrt64(rR * iL), idn = rcp64(1.0 + Dr);
+  double ut2, utn;
+#pragma unroll
+  for (int j = 0; j < D; ++j) {
+    const double ut = fma(vR[j], Dr, vL[j]) * idn;
+    ut2 = j ? fma(ut, ut, ut2) : ut * ut;
+    utn = j ? fma(ut, n[j], utn) : ut * n[j];
+  }
+  const double Ht = fma(HR, Dr, HL) * idn, ct = sqrt64(gm1 * fma(-0.5, ut2, Ht));
+  const double sl1 = unL - cL, sl2 = utn - ct, sr1 = unR + cR, sr2 = utn + ct;
+  const double SL = less64(sl1, sl2) ? sl1 : sl2, SR = less64(sr1, sr2) ? sr2 : sr1;
+  const double aL = SL - unL, aR = SR - unR, mL = rL * aL, mR = rR * aR;
+  const double SM = (fma(mR, unR, -(mL * unL)) + (pL - pR)) * rcp64(mR - mL);
+  // the cases in the order SL > 0, SM > 0, SR > 0, else, without branches (see hllc)
+  const bool cl = positive64(SL), cm = positive64(SM), cr = positive64(SR);
+  const bool left = cl || cm, sup = cl || (!cm && !cr);
+  double uk[NV];
+#pragma unroll
+  for (int v = 0; v < NV; ++v) uk[v] = left ? uL[v] : uR[v];
+  const double pk = left ? pL : pR, unk = left ? unL : unR, Sk = left ? SL : SR, ak = left ? aL : aR;
+  F[0] = uk[0] * unk;
+#pragma unroll
+  for (int j = 0; j < D; ++j) F[1 + j] = fma(uk[1 + j], unk, pk * n[j]);
+  F[NV - 1] = (uk[NV - 1] + pk) * unk;
+  const double ps = fma(-mL, unL - SM, pL);
+  const double fct = rcp64(Sk - SM), s1 = fma(ak, fct, -1.0), dp = (ps - pk) * fct;
+  double G[NV];  // S_k (U* - U)
+  G[0] = Sk * (s1 * uk[0]);
+#pragma unroll
+  for (int j = 0; j < D; ++j) G[1 + j] = Sk * fma(dp, n[j], s1 * uk[1 + j]);
+  G[NV - 1] = Sk * fma(fma(ps, SM, -(pk * unk)), fct, s1 * uk[NV - 1]);
+#pragma unroll
+  for (int v = 0; v < NV; ++v) F[v] = sup ? F[v] : F[v] + G[v];
+}
+
+// Local CFL step |V_i| / sum_f |A_f| (|u_i . n_f| + c_i) of the FP64 path: the velocity and the speed
+// of sound of a state, a face's term, and the step from their sum in face order. Every rounding is
+// written out: the set-state kernels and the stage update must give the same bits.
+template <int D>
+__device__ __forceinline__ void speeds64(const double *u, const double g, double (&vel)[D], double &c) {
+  const double ir = rcp64(u[0]);
+  double ke = 0.0;
+#pragma unroll
+  for (int j = 0; j < D; ++j) {
+    vel[j] = __dmul_rn(u[1 + j], ir);
+    ke = fma(u[1 + j], vel[j], ke);
+  }
+  c = sqrt64(__dmul_rn(__dmul_rn(g, __dmul_rn(g - 1.0, fma(-0.5, ke, u[D + 1]))), ir));
+}
+template <int D>
+__device__ __forceinline__ double face_speed64(const double *gf, const double (&vel)[D], const double c) {
+  double un = 0.0;
+#pragma unroll
+  for (int j = 0; j < D; ++j) un = fma(vel[j], gf[j], un);
+  return __dmul_rn(gf[3], __dadd_rn(fabs(un), c));
+}
+template <int D>
+__device__ __forceinline__ double local_dt64(const KArgs &a, const int64_t i, const double *u) {
+  double vel[D], c, s = 0.0;
+  speeds64<D>(u, a.gamma, vel, c);
+#pragma unroll
+  for (int f = 0; f <= D; ++f) s = __dadd_rn(s, face_speed64<D>(a.geo + (i * (D + 1) + f) * 4, vel, c));
+  return rcp64(__dmul_rn(s, a.vol[i]));
+}
+
+template <int D, int NQ>
+__global__ void __launch_bounds__(256) face_flux64_kernel(const KArgs a) {
+  constexpr int NV = D + 2, NVP = Lay<D>::NVP, NF = D + 1, NFP = (NV + 3) & ~3;
+  constexpr int FPW = 32 / NQ;  // faces of a warp; two spare lanes with three points a face
+  pdl_wait(a);                  // face states of the reconstruction
+  const int lane = threadIdx.x & 31, grp = lane / NQ, q = lane - grp * NQ, base = grp * NQ;
+  const int64_t face = ((int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * FPW + grp;
+  const bool active = grp < FPW && face < a.nfaces;
+  const int64_t e = active ? face : a.nfaces - 1;  // spare lanes shadow a face and store nothing
+  const int2 codes = __ldg(reinterpret_cast<const int2 *>(a.face) + e);  // owner, neighbour side
+  const int64_t i = codes.x >> 2;
+  const int f = codes.x & 3;
+  const double *__restrict__ Uf = (const double *)a.Uf;
+  auto state = [&](int64_t cell, int face_of, double *u) {
+    const double *p = Uf + ((cell * NF + face_of) * NQ + q) * NV;
+    if constexpr (D == 2) {
+      load16<double, NV>(p, u);
+    } else {
+#pragma unroll
+      for (int v = 0; v < NV; ++v) u[v] = __ldg(p + v);
+    }
+  };
+  double gf[4], uI[NV], uO[NV], F[NV];
+  load16<double, 4>(a.geo + (i * NF + f) * 4, gf);
+  state(i, f, uI);
+  if (codes.y >= 0) {
+    state(codes.y >> 2, codes.y & 3, uO);
+  } else {  // boundary face: its kind's outside state
+    double um[NVP];
+#pragma unroll
+    for (int v = 0; v < NVP; ++v) um[v] = a.U[i * NVP + v];
+    boundary_state<D, double, 1>(a, i, (__ldg(a.fmeta + i) >> (kMetaKindShift + 2 * f)) & 3u, gf, uI, um, uO);
+  }
+  hllc64<D>(uI, uO, gf, a.gamma, F);
+  double w = a.fw[0];
+#pragma unroll
+  for (int t = 1; t < NQ; ++t) w = (q == t) ? a.fw[t] : w;
+  w *= gf[3];
+  double out[NFP];
+#pragma unroll
+  for (int v = 0; v < NFP; ++v) {
+    double x = 0.0;
+    if (v < NV) {
+      x = w * F[v];
+      if constexpr (NQ == 3) {
+        const double y = __shfl_sync(0xffffffffu, x, base + 1), z = __shfl_sync(0xffffffffu, x, base + 2);
+        x = (x + y) + z;  // the face's first lane stores it
+      } else {
+#pragma unroll
+        for (int o = 1; o < NQ; o <<= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+      }
+    }
+    out[v] = x;
+  }
+  if (active && q == 0) store16<double, NFP>((double *)a.Ff + e * NFP, out);
+}
+
+template <int D>
+__global__ void __launch_bounds__(256) cell_update64_kernel(const KArgs a) {
+  constexpr int NV = D + 2, NVP = Lay<D>::NVP, NF = D + 1, NFP = (NV + 3) & ~3, CPW = 32 / NV;
+  pdl_wait(a);  // the face fluxes of this stage
+  const int lane = threadIdx.x & 31, grp = lane / NV, v = lane - grp * NV, base = grp * NV;
+  const int64_t N = a.N;
+  const int64_t cell = ((int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * CPW + grp;
+  const bool active = grp < CPW && cell < N;
+  const int64_t i = active ? cell : N - 1;  // spare lanes shadow a cell and store nothing
+  const int4 cf4 = __ldg(reinterpret_cast<const int4 *>(a.cellface) + i);
+  const int cf[4] = {cf4.x, cf4.y, cf4.z, cf4.w};
+  const int64_t at = i * NVP + v;
+  const double u = a.U[at];
+  double acc = 0.0;  // sum_f |A_f| sum_q w_q F_q, signed for this cell
+#pragma unroll
+  for (int f = 0; f < NF; ++f) {
+    const double x = __ldg((const double *)a.Ff + (int64_t)(cf[f] & 0x7FFFFFFF) * NFP + v);
+    acc += cf[f] < 0 ? -x : x;
+  }
+  const int mesh = (a.nmesh > 1) ? mesh_of(a, i) : 0;
+  const double dtv = a.dt[mesh] * a.vol[i];  // dt / |V_i|
+  double r, ac = 0.0;
+  if (!a.rk4) {  // SSP-RK3 (Shu-Osher), as stage_tail
+    r = fma(-dtv, acc, u);
+    if (a.stage == 1) r = 0.75 * a.Un[at] + 0.25 * r;
+    else if (a.stage == 2) r = (1.0 / 3.0) * a.Un[at] + (2.0 / 3.0) * r;
+  } else {       // classical RK4 with its running sum, as stage_tail
+    const double F = -dtv * acc;  // dt k_s
+    const double w = (a.stage == 0 || a.stage == 3) ? 1.0 / 6.0 : 1.0 / 3.0;
+    ac = fma(F, w, a.stage == 0 ? u : a.Acc[at]);
+    r = a.stage == 3 ? ac : (a.stage == 0 ? u : a.Un[at]) + (a.stage == 2 ? F : 0.5 * F);
+  }
+  const bool finite = finite64(r);
+  if (active) {
+    if (a.stage == 0) a.Un[at] = u;
+    if (a.rk4 && a.stage < 3) a.Acc[at] = ac;
+    a.U[at] = r;
+    if (!finite) atomicOr(a.err, kErrNonFinite);
+  }
+  if (a.stage == a.last_stage) {  // the CFL step of the next step: lane f takes face f
+    double full[NV], vel[D], c, s = 0.0;
+    bool fin = active;
+#pragma unroll
+    for (int t = 0; t < NV; ++t) {
+      full[t] = __shfl_sync(0xffffffffu, r, base + t);
+      fin = fin && finite64(full[t]);
+    }
+    speeds64<D>(full, a.gamma, vel, c);
+    double gf[4];
+    load16<double, 4>(a.geo + (i * NF + min(v, NF - 1)) * 4, gf);
+    const double x = face_speed64<D>(gf, vel, c);
+#pragma unroll
+    for (int f = 0; f < NF; ++f) s = __dadd_rn(s, __shfl_sync(0xffffffffu, x, base + f));
+    const double dt = a.cfl * rcp64(__dmul_rn(s, a.vol[i]));
+    warp_min_to(a.dt, a.nmesh + mesh, fin ? dt : 1e300);
+  }
+}
+
+}  // namespace
+}  // namespace cteno

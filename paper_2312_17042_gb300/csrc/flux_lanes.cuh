@@ -10,12 +10,12 @@
 namespace cteno {
 namespace {
 
-template <int D, typename T, int NQ>
+template <int D, int NQ>
 __global__ void __launch_bounds__(256) flux_lanes_kernel(const KArgs a) {
   using L = Lay<D>;
   constexpr int NV = L::NV, NVP = L::NVP, NF = L::NF, FB = NQ * NV;
   constexpr int CPW = 32 / NF;
-  constexpr bool F32 = sizeof(T) == 4;
+  using T = float;
   pdl_wait(a);
   const int lane = threadIdx.x & 31;
   const int grp = lane / NF;
@@ -26,9 +26,8 @@ __global__ void __launch_bounds__(256) flux_lanes_kernel(const KArgs a) {
   const bool active = grp < CPW && cell < N;
   const int64_t i = active ? cell : N - 1;  // spare lanes shadow a valid cell, store nothing
   const T *__restrict__ Uf = (const T *)a.Uf;
-  const T *__restrict__ G = F32 ? (const T *)a.geo32 : (const T *)a.geo;
-  T g;
-  if constexpr (F32) g = a.gamma32; else g = a.gamma;
+  const T *__restrict__ G = a.geo32;
+  const T g = a.gamma32;
   const uint32_t meta = __ldg(a.fmeta + i);
   const int64_t j = __ldg(a.nbr + i * 4 + f);
   const int fj = (meta >> (2 * f)) & 3u;
@@ -51,10 +50,9 @@ __global__ void __launch_bounds__(256) flux_lanes_kernel(const KArgs a) {
 #pragma unroll
   for (int q = 0; q < NQ; ++q) {
     T F[NV];
-    if (own) hllc<D, T>(uI + q * NV, uO + q * NV, n, g, F);
-    else hllc<D, T>(uO + q * NV, uI + q * NV, n, g, F);
-    T w;
-    if constexpr (F32) w = a.fw32[q]; else w = a.fw[q];
+    if (own) hllc<D>(uI + q * NV, uO + q * NV, n, g, F);
+    else hllc<D>(uO + q * NV, uI + q * NV, n, g, F);
+    const T w = a.fw32[q];
 #pragma unroll
     for (int v = 0; v < NV; ++v) Ff[v] = (q == 0) ? w * F[v] : Ff[v] + w * F[v];
   }
@@ -73,22 +71,16 @@ __global__ void __launch_bounds__(256) flux_lanes_kernel(const KArgs a) {
   for (int v = 0; v < NVP; ++v) res[v] = 0.0;
 #pragma unroll
   for (int v = 0; v < NV; ++v) {
-    double acc = 0.0;
-    float hi = 0.0f, lo = 0.0f;
-    if constexpr (F32) {  // exact FP32 accumulation over the faces, as in the per-cell kernel
+    float hi = 0.0f, lo = 0.0f;  // exact FP32 accumulation over the faces, as in the per-cell kernel
 #pragma unroll
-      for (int ff = 0; ff < NF; ++ff) {
-        float s, e;
-        two_sum(hi, __shfl_sync(0xffffffffu, contrib[v], base + ff), s, e);
-        hi = s;
-        lo += e;
-      }
-    } else {
-#pragma unroll
-      for (int ff = 0; ff < NF; ++ff) acc += (double)__shfl_sync(0xffffffffu, contrib[v], base + ff);
+    for (int ff = 0; ff < NF; ++ff) {
+      float s, e;
+      two_sum(hi, __shfl_sync(0xffffffffu, contrib[v], base + ff), s, e);
+      hi = s;
+      lo += e;
     }
     if (v % NF == f) {  // FP64 work only in the lane that updates variable v
-      if constexpr (F32) acc = f32_to_f64(hi) + f32_to_f64(lo);
+      const double acc = f32_to_f64(hi) + f32_to_f64(lo);
       const double u = a.U[i * NVP + v];
       double r, s4 = 0.0;
       if (!a.rk4) {  // SSP-RK3 (Shu-Osher), as stage_tail
@@ -117,7 +109,7 @@ __global__ void __launch_bounds__(256) flux_lanes_kernel(const KArgs a) {
         if (a.stage == 0) a.Un[i * NVP + v] = u;
         if (a.rk4 && a.stage < 3) a.Acc[i * NVP + v] = s4;
         a.U[i * NVP + v] = r;
-        if (a.U32) reinterpret_cast<float2 *>(a.U32)[i * NVP + v] = f64_split(r);
+        reinterpret_cast<float2 *>(a.U32)[i * NVP + v] = f64_split(r);
       }
     }
   }
@@ -133,11 +125,8 @@ __global__ void __launch_bounds__(256) flux_lanes_kernel(const KArgs a) {
     for (int v = 0; v < NV; ++v) fin = fin && finite64(full[v]);
     T ft[NVP];
 #pragma unroll
-    for (int v = 0; v < NVP; ++v) {
-      if constexpr (F32) ft[v] = f64_split(full[v]).x;
-      else ft[v] = full[v];
-    }
-    warp_min_to(a.dt, a.nmesh + mesh, fin ? a.cfl * local_dt<D, T>(a, i, ft) : 1e300);
+    for (int v = 0; v < NVP; ++v) ft[v] = f64_split(full[v]).x;
+    warp_min_to(a.dt, a.nmesh + mesh, fin ? a.cfl * local_dt<D>(a, i, ft) : 1e300);
   }
 }
 
