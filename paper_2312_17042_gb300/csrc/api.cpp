@@ -11,7 +11,7 @@
 #include <vector>
 
 #include "device.h"
-#include "fixed.h"
+#include "tiles.h"
 #include "internal.h"
 
 using namespace cteno;
@@ -547,8 +547,10 @@ int cteno_lsq_build(cteno_ctx *ctx) {
   CK(dalloc(ctx, &ctx->nbr, sizeof(int32_t) * 4 * N));
   CK(dalloc(ctx, &ctx->cinfo, sizeof(uint32_t) * N));
   CK(dalloc(ctx, &ctx->fmeta, sizeof(uint32_t) * N));
-  const bool fixed = !ctx->fp32 && !ctx->p.characteristic;  // operators as integers (fixed.h)
-  CK(dalloc(ctx, &ctx->Pc, sT * ctx->nk * M * (fixed ? fixed_cells(d, N) : N)));
+  // conserved variables: FP64 operators as integers, degrees 4 to 6 in FP32, in tiles (tiles.h)
+  const bool fixed = !ctx->fp32 && !ctx->p.characteristic;
+  const bool tiled = fixed || (ctx->p.degree >= 4 && !ctx->p.characteristic);
+  CK(dalloc(ctx, &ctx->Pc, sT * ctx->nk * M * (tiled ? tiled_cells(d, N) : N)));
   CK(dalloc(ctx, &ctx->Pd, sT * nf * pds * N));
   std::vector<int32_t> hphi;  // the face table, rows of an even number of entries
   if (fixed) {
@@ -626,6 +628,7 @@ int cteno_lsq_build(cteno_ctx *ctx) {
   s.Pc = ctx->Pc;
   s.Pd = ctx->Pd;
   s.Pe = ctx->Pe;
+  s.tiled = tiled;
   s.store_fp32 = ctx->fp32 ? 1 : 0;
   s.geo = ctx->geo;
   s.vol = ctx->vol;
@@ -1072,9 +1075,7 @@ int cteno_autotune(cteno_ctx *ctx, int32_t *best_out) {
   for (int b : {128, 256}) cand.push_back(kLaneSchedule + b);
   std::vector<int> rcand = cand;
   if (!ctx->fp32) rcand = {64, 128, 256};  // the FP64 path has one reconstruction schedule
-  if (ctx->p.degree >= 4) rcand = {kLaneSchedule + 64, kLaneSchedule + 128, kLaneSchedule + 256};
-  if (ctx->p.degree >= 4 && ctx->fp32 && !ctx->p.characteristic)
-    for (int b : {64, 128, 256}) rcand.push_back(kHighOcc + b);
+  if (ctx->p.degree >= 4) rcand = {kLaneSchedule + 32, kLaneSchedule + 64, kLaneSchedule + 128};
   // the staged schedules (mixed path) whose two stages fit
   if (ctx->fp32 && ctx->p.degree <= 3)
     for (int b : {kStagedCells + 32, kStagedCells + 64, kStagedCells + 128, kStagedLanes + 64,

@@ -78,10 +78,11 @@ struct DevTables {
 //   U, Un   double [N][NVP]        conserved means (padding entries unused)
 //   U32     float2 [N][NVP]        mixed path: (hi, lo) = (fl32(U), fl32(U - hi))
 //   st      int32  [N][M]          stencil ids, directional members first (face after face)
-//   Pc      T      [N][M][nk]      central pseudo-inverse, member-major
+//   Pc      T      [N][M][nk]      central pseudo-inverse, member-major; in tiles (tiles.h) on the FP64
+//                                  path and at degrees 4 to 6, conserved variables
 //   Pd      T      [N][NF][PDS]    directional pseudo-inverses (layout of Dir<D, R>)
 //           FP64 path, conserved variables: Pc and Pd hold int2 (h, l), entries of 57-bit integers
-//           (layout in fixed.h)
+//           (layout in tiles.h)
 //   Pe      int8   [N][kFixExp]    block exponents of those: rows of Pc, then faces of Pd
 //   Uf      T      [N][NF][NQ][NV] face Gauss-point states
 //   nbr     int32  [N][4]          face neighbours, -1 on a boundary
@@ -101,7 +102,7 @@ struct KArgs {
   const void *Pc;
   const void *Pd;
   const int8_t *Pe;
-  const int2 *phifx;        // FP64 path: the face table (FixShape)
+  const int2 *phifx;        // FP64 path: the face table (TileShape)
   void *Uf;
   uint8_t *flags;
   const int32_t *nbr;
@@ -173,6 +174,7 @@ struct SetupArgs {
   double period[3];
   void *Pc, *Pd;            // outputs, T = double (FP64 path) or float (mixed path)
   int store_fp32;
+  int tiled;                // Pc in the layout of tiles.h
   int8_t *Pe;               // not null: Pc, Pd as 57-bit integers, Pe their exponents
   double *geo, *vol;       // vol receives 1 / |V_i|
   float *geo32;
@@ -276,8 +278,7 @@ inline long long recon_staged_smem(int d, int degree, int fp32, int block) {
 void launch_setup(int dim, int degree, const SetupArgs &a, cudaStream_t s);
 // Central degrees 4 to 6 (2D): constant banks and the variable-per-lane reconstruction
 // (recon_2d_high.cu); launch values other than kLaneSchedule + b (and, on the mixed path without
-// the characteristic projection, kHighOcc + b: the same schedule compiled for at most 64
-// registers per thread) give cudaErrorInvalidValue.
+// the characteristic projection, kHighOcc + b, the same kernel) give cudaErrorInvalidValue.
 constexpr int kHighOcc = 1536;
 cudaError_t upload_recon_tables_2d_high(int degree, const Tables &t, cudaStream_t s);
 cudaError_t launch_recon_2d_high(int degree, int fp32, int scheme, const KArgs &a, int block, cudaStream_t s);

@@ -6,7 +6,7 @@ namespace {
 
 template <int D, int R, int SCHEME>
 cudaError_t launch_fixed(const KArgs &a, int threads, cudaStream_t s) {
-  using S = FixShape<D, R>;
+  using S = TileShape<D, R, 8>;
   threads = std::min(threads, 128);  // the kernel's block: 4 warps at most
   const int64_t cells = (int64_t)(threads / 32) * S::CPW;
   const unsigned grid = (unsigned)((a.N + cells - 1) / cells);

@@ -21,7 +21,7 @@
 // where they hold by a margin far above its error, and in FP64 as printed elsewhere.
 //
 // Schedule: variable per lane, as recon_lane, one tile per warp. The operators stream through the warp's
-// ring of shared-memory stages, one bulk copy per chunk (fixed.h), issued before the previous kernel has
+// ring of shared-memory stages, one bulk copy per chunk (tiles.h), issued before the previous kernel has
 // ended: read from global memory they cost twice the time, at 8 to 16 warps per SM. The
 // differences of the directional members (the first slots of the stencil list) wait in shared
 // memory between the two products.
@@ -31,8 +31,8 @@
 // 2D degree 5, 4200 cells 81 -> 37 us; 2D degree 2, 2048 cells 19 (51 in blocks of 128) -> 13 us.
 #pragma once
 
-#include "fixed.h"
 #include "recon.cuh"
+#include "tiles.h"
 
 namespace cteno {
 
@@ -163,16 +163,9 @@ __device__ __forceinline__ bool select_sure(const KArgs &a, const float SI0, con
   return sure;
 }
 
-// Blocks of 4 warps an SM is to hold (register cap): what shared memory allows, at most 4.
-template <int D, int R>
-struct FixBlocks {
-  static constexpr int fit = 227 * 1024 / (FixShape<D, R>::PHI_BYTES + 16 + 4 * FixShape<D, R>::WARP_BYTES + 1024);
-  static constexpr int value = fit < 4 ? fit : 4;
-};
-
 template <int D, int R, int SCHEME>
-__global__ void __launch_bounds__(128, FixBlocks<D, R>::value) recon_fixed_kernel(const KArgs a) {
-  using S = FixShape<D, R>;
+__global__ void __launch_bounds__(128, TileShape<D, R, 8>::BLOCKS) recon_fixed_kernel(const KArgs a) {
+  using S = TileShape<D, R, 8>;
   constexpr int NV = S::NV, NVP = S::NVP, NF = S::NF, NK = S::NK, M = S::M, NQ = S::NQ, NP = S::NP;
   constexpr int KD = S::KD, ND = S::ND, PDS = S::PDS, G = S::G, SLOTS = S::SLOTS, CPW = S::CPW;
   constexpr int MC = S::MC, NCH = S::NCH, NST = S::NST, NKP = S::NKP;

@@ -4,7 +4,7 @@
 // directional polynomials of degree 2 (5 unknowns, at most 10 members each, within the central
 // stencil), and n-point Gauss-Legendre edges (n = 3, 3, 4).
 //
-// Variable-per-lane schedule only: a group of four lanes reconstructs one cell, lane v conserved
+// Variable-per-lane schedule: a group of four lanes reconstructs one cell, lane v conserved
 // variable v, and keeps its own 27 + 15 coefficients at most (a thread holding all four variables
 // would need four times that in registers). The steps are those of recon.cuh (eqs. 10-23,
 // Alg. 1 / 2, CWENO and TENO weightings):
@@ -19,6 +19,7 @@
 #pragma once
 
 #include "recon.cuh"
+#include "tiles.h"
 
 namespace cteno {
 
@@ -102,9 +103,9 @@ inline cudaError_t upload_high_tables(const Tables &t, cudaStream_t s) {
   return cudaStreamSynchronize(s);  // the host arrays above go out of scope
 }
 
-// One block of 8-cell warps; lane v of group grp reconstructs variable v of cell 8 w + grp (the
+// The characteristic reconstruction: one block of 8-cell warps; lane v of group grp reconstructs variable v of cell 8 w + grp (the
 // last cell shadows the lanes past the end and stores nothing).
-template <int R, typename T, int SCHEME, bool CHR>
+template <int R, typename T, int SCHEME>
 __device__ __forceinline__ void recon_high_body(const KArgs &a) {
   using H = HighShape<R>;
   using DR = Dir<2, R>;
@@ -207,7 +208,7 @@ __device__ __forceinline__ void recon_high_body(const KArgs &a) {
     return s;
   };
   auto phi = [](int f, int q, int k) { return cPhiH<T, R>((f * NQ + q) * NK + k); };
-  lane_faces<2, NK, KD, NQ, T, SCHEME, CHR>(a, i, active, v, base, ao, ad, info, U0, L0, oc, sid,
+  lane_faces<2, NK, KD, NQ, T, SCHEME, true>(a, i, active, v, base, ao, ad, info, U0, L0, oc, sid,
                                            phi_tab(phi));
   // CFL time step bookkeeping at the first stage of a step: dt[next] -> dt[cur]
   if (a.dt_swap && blockIdx.x == 0)
@@ -217,17 +218,155 @@ __device__ __forceinline__ void recon_high_body(const KArgs &a) {
     }
 }
 
-template <int R, typename T, int SCHEME, bool CHR>
+template <int R, typename T, int SCHEME>
 __global__ void __launch_bounds__(256) recon_high_kernel(const KArgs a) {
-  recon_high_body<R, T, SCHEME, CHR>(a);
+  recon_high_body<R, T, SCHEME>(a);
 }
 
-// The FP32 body compiled for at most 64 registers per thread (launch value kHighOcc + b): 32
-// resident warps per SM instead of 24-28, for a kernel that waits on its record loads and
-// neighbour gathers (a few dozen bytes of spill).
+// Conserved variables on the mixed path: the same steps and the same order of every sum, one 8-cell tile
+// per warp, the operators streamed through the warp's shared memory (tiles.h): one bulk copy per
+// chunk and one for the directional operators, issued before the previous kernel has ended; the means of
+// the next group of members are gathered while a group is multiplied, and the differences of the
+// directional members (the first slots of the list) wait in shared memory. Reading the records with
+// per-lane loads instead left the kernel waiting for them (22 of 26 stall cycles per issue): bound by
+// latency at 45 % of the memory rate.
 template <int R, int SCHEME>
-__global__ void __launch_bounds__(256, 4) recon_high_kernel_occ(const KArgs a) {
-  recon_high_body<R, float, SCHEME, false>(a);
+__global__ void __launch_bounds__(128, TileShape<2, R, 4>::BLOCKS) recon_high_stream_kernel(const KArgs a) {
+  using S = TileShape<2, R, 4>;
+  constexpr int NV = 4, NVP = 4, NF = 3, NK = S::NK, M = S::M, NQ = S::NQ, KD = S::KD, ND = S::ND;
+  constexpr int NDP = Dir<2, R>::NDP, PDS = S::PDS, MC = S::MC, NCH = S::NCH, NST = S::NST, SLOTS = S::SLOTS;
+  extern __shared__ __align__(128) unsigned char smem[];
+  unsigned char *const wmem = smem + (threadIdx.x >> 5) * S::WARP_BYTES;
+  float *const sdel = reinterpret_cast<float *>(wmem + S::HDR + NST * S::STAGE) + (threadIdx.x & 31);
+  uint64_t *const bar = reinterpret_cast<uint64_t *>(wmem + S::HDR + NST * S::STAGE + S::DELTA);  // header, stages
+  const int lane = threadIdx.x & 31, grp = lane / NV, v = lane - grp * NV, base = grp * NV;
+  const int64_t N = a.N;
+  const int64_t tile = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), c0 = tile * S::CPW;
+  const int n = (int)max((int64_t)0, min((int64_t)S::CPW, N - c0));  // the warp's cells
+  auto issue = [&](int c) {  // lane 0: chunk c of the warp's tile
+    uint64_t *b = &bar[1 + c % NST];
+    mbar_arrive_expect_tx(b, S::STAGE);
+    bulk_copy_g2s(wmem + S::HDR + (c % NST) * S::STAGE, (const unsigned char *)a.Pc + (tile * NCH + c) * S::STAGE,
+                  S::STAGE, b);
+  };
+  if (lane == 0 && n > 0) {
+    for (int b = 0; b < 1 + NST; ++b) mbar_init(&bar[b], 1);
+    fence_barrier_init();
+    for (int c = 0; c < NST; ++c) issue(c);
+    mbar_arrive_expect_tx(&bar[0], (uint32_t)(n * NF * PDS * 4));
+    bulk_copy_g2s(wmem, (const float *)a.Pd + c0 * (NF * PDS), (uint32_t)(n * NF * PDS * 4), &bar[0]);
+  }
+  __syncwarp();
+  pdl_wait(a);  // the state written by the previous stage's update
+  if (a.dt_swap && blockIdx.x == 0)  // the CFL step: dt[next] -> dt[cur]
+    for (int t = threadIdx.x; t < a.nmesh; t += blockDim.x) {
+      a.dt[t] = a.dt[a.nmesh + t];
+      a.dt[a.nmesh + t] = 1e300;
+    }
+  if (n == 0) return;  // a warp past the last cell
+  // a bounded wait of the whole warp for its copies; on a timeout the warp reports it, gives the
+  // copies in flight (chunks c up to `last`) a second bounded wait and stops
+  auto arrived = [&](uint64_t *b, uint32_t parity, int c, int last) {
+    const bool ok = mbar_wait(b, parity, kStageWaitNs);
+    if (!__any_sync(0xffffffffu, !ok)) return true;
+    if (lane == 0) {
+      atomicOr(a.err, kErrTimeout);
+      mbar_wait(&bar[0], 0, kStageWaitNs);
+      for (; c < last; ++c) mbar_wait(&bar[1 + c % NST], (uint32_t)((c / NST) & 1), kStageWaitNs);
+    }
+    __syncwarp();
+    return false;
+  };
+  const bool active = grp < n;
+  const int slot = active ? grp : n - 1;  // spare lanes shadow a valid cell and store nothing
+  const int64_t i = c0 + slot;
+  const float2 *__restrict__ Uv = reinterpret_cast<const float2 *>(a.U32) + v;
+  const int32_t *__restrict__ sti = a.st + i * M;
+  const float2 own = __ldg(Uv + i * NVP);
+  const float U0 = own.x, L0 = own.y;
+  float2 nx[MC];  // the next chunk's member means
+  auto fetch = [&](int c) {
+#pragma unroll
+    for (int g = 0; g < MC; g += 2) {
+      const int2 j = __ldg(reinterpret_cast<const int2 *>(sti + c * MC + g));
+      nx[g] = __ldg(Uv + (int64_t)j.x * NVP);
+      nx[g + 1] = __ldg(Uv + (int64_t)j.y * NVP);
+    }
+  };
+  fetch(0);
+  const uint32_t info = __ldg(a.cinfo + i);
+  float ao[NK];
+#pragma unroll
+  for (int k = 0; k < NK; ++k) ao[k] = 0.0f;
+#pragma unroll 1
+  for (int c = 0; c < NCH; ++c) {
+    float du[MC];
+#pragma unroll
+    for (int g = 0; g < MC; ++g) {
+      du[g] = (nx[g].x - U0) + (nx[g].y - L0);
+      if (c * MC + g < SLOTS) sdel[(c * MC + g) * 32] = du[g];
+    }
+    if (c + 1 < NCH) fetch(c + 1);
+    if (!arrived(&bar[1 + c % NST], (uint32_t)((c / NST) & 1), c, min(c + NST, NCH))) return;
+    const float *__restrict__ P =
+        reinterpret_cast<const float *>(wmem + S::HDR + (c % NST) * S::STAGE) + slot * (MC * NK);
+    float pb[4];
+#pragma unroll
+    for (int e = 0; e < MC * NK; ++e) {
+      if (e % 4 == 0) load16<float, 4, true>(P + e, pb);
+      ao[e % NK] += pb[e % 4] * du[e / NK];
+    }
+    if (NST < NCH && c + NST < NCH) {
+      __syncwarp();  // every lane is done with this stage
+      if (lane == 0) {
+        fence_proxy_async_shared();
+        issue(c + NST);
+      }
+    }
+  }
+  // directional coefficients (degree 2): the members of face f are the next slots of the list
+  if (!arrived(&bar[0], 0, NCH, NCH)) return;
+  const uint32_t adm = (info >> kInfoAdmShift) & 7u;
+  const float *__restrict__ Pdi = reinterpret_cast<const float *>(wmem) + slot * (NF * PDS);
+  float ad[NF][KD];
+  {
+    int off = 0;
+#pragma unroll
+    for (int f = 0; f < NF; ++f) {
+      const int nm = (info >> (4 * f)) & 15u;
+#pragma unroll
+      for (int k = 0; k < KD; ++k) ad[f][k] = 0.0f;
+      if ((adm >> f) & 1u) {
+        float du[ND];
+#pragma unroll
+        for (int j = 0; j < ND; ++j) du[j] = (j < nm) ? sdel[(off + j) * 32] : 0.0f;
+#pragma unroll
+        for (int k = 0; k < KD; ++k) {
+          float pk[NDP];
+          load16<float, NDP, true>(Pdi + f * PDS + k * NDP, pk);
+          float s = 0.0f;
+#pragma unroll
+          for (int j = 0; j < ND; ++j) s += pk[j] * du[j];
+          ad[f][k] = s;
+        }
+      }
+      off += nm;
+    }
+  }
+  auto oc = [](int idx) { return cOH<float, R>(idx); };
+  auto sid = [](const float (&adf)[KD]) {
+    float s = 0.0f;
+#pragma unroll
+    for (int k = 0; k < KD; ++k) {
+      float rr = 0.0f;
+#pragma unroll
+      for (int l = k; l < KD; ++l) rr += cOH<float, R>(k * NK + l) * adf[l];
+      s += adf[k] * rr;
+    }
+    return s;
+  };
+  auto phi = [](int f, int q, int k) { return cPhiH<float, R>((f * NQ + q) * NK + k); };
+  lane_faces<2, NK, KD, NQ, float, SCHEME, false>(a, i, active, v, base, ao, ad, info, U0, L0, oc, sid, phi_tab(phi));
 }
 
 }  // namespace cteno

@@ -3,7 +3,7 @@
 // least-squares matrices and the pseudo-inverses P = R^-1 Q^T diag(|V'_m|), so that the
 // coefficients of eq. 12 are a = P (U_m - U_0). One thread per cell; run once per mesh set.
 #include "device.h"
-#include "fixed.h"
+#include "tiles.h"
 
 namespace cteno {
 namespace {
@@ -296,7 +296,7 @@ __global__ void __launch_bounds__(128) setup_kernel(const SetupArgs a) {
   double dg[NK], vt[NK], bt[NK];
   if (!householder<NK>(W, M, NK, dg, vt, bt)) atomicOr(a.err, kErrRank);
   if (a.Pe) {  // FP64 path: rows in the orthonormal basis, written as FP64 first, then scaled in place
-    using FX = FixShape<D, R>;
+    using FX = TileShape<D, R, 8>;
     double top[NK], *P = (double *)a.Pc;
     for (int k = 0; k < NK; ++k) top[k] = 0.0;
     for (int p = 0; p < M; ++p) {
@@ -323,7 +323,9 @@ __global__ void __launch_bounds__(128) setup_kernel(const SetupArgs a) {
     double col[NK];
     pinv_column<NK, M>(W, M, NK, dg, vt, bt, p, col);
     for (int k = 0; k < NK; ++k) {
-      const int64_t idx = (i * M + p) * NK + k;
+      int64_t idx = (i * M + p) * NK + k;
+      if constexpr (DR::HIGH)
+        if (a.tiled) idx = TileShape<D, R, 4>::index(i, p, k);
       if (a.store_fp32)
         ((float *)a.Pc)[idx] = (float)(col[k] * Vp[p]);
       else

@@ -1,0 +1,59 @@
+// tiles.h -- layout of the least-squares operators that a warp streams through shared memory (written by
+// setup.cu; read by recon_fixed.cuh, the FP64 path, and recon_high.cuh, the mixed path's degrees 4 to 6).
+//
+// The cells are taken in tiles of CPW, the cells of one warp of the reconstruction, and a tile's
+// central rows in chunks of MC members, so that the chunk a warp copies is one contiguous span:
+//   Pc  [tile][M / MC][CPW][MC][NK]   (the last tile is allocated whole)
+//   Pd  [cell][face][PDS]             (Dir<D, R>; FP64 path: member-major j * KD + k at every degree)
+// Entries (E bytes): float, or on the FP64 path int2 (h, l), the integer h 2^29 + l of 57 bits and a
+// sign in units of 2^(e - 57), e the exponent of its block (KArgs::Pe).
+#pragma once
+
+#include <cstdint>
+
+#include "device.h"
+
+namespace cteno {
+
+template <int D, int R, int E>
+struct TileShape {
+  static constexpr int NV = D + 2, NVP = Lay<D>::NVP, NF = D + 1;
+  static constexpr int NK = (D == 2 ? (R + 1) * (R + 2) / 2 : (R + 1) * (R + 2) * (R + 3) / 6) - 1;
+  static constexpr int M = 2 * (NK + 1);
+  static constexpr int NQ = D == 3 ? 4 : (R + 2) / 2 > 2 ? (R + 2) / 2 : 2;
+  static constexpr int KD = Dir<D, R>::KD, ND = Dir<D, R>::ND, PDS = Dir<D, R>::PDS;
+  static constexpr int CPW = 32 / NV;
+  // Chunks of the central record, NST of them in flight, and the members whose differences are formed
+  // together. FP64: all of it up to 20 members (2D degrees 2, 3; 3D degree 2). Mixed: chunks of 4.4,
+  // 3.8 and 6.9 kB a warp at degrees 4, 5 and 6, 12 to 15 kB in flight, which with 11 to 12 warps covers
+  // the memory latency of an SM (about 45 kB at the full rate) through the arithmetic of each warp.
+  static constexpr int MC = E == 4 ? (R == 4 ? 10 : R == 5 ? 6 : 8) : M <= 20 ? M : M % 4 == 0 ? 4 : 6;
+  static constexpr int NCH = M / MC, NMAX = E == 4 ? (R == 4 ? 3 : R == 5 ? 4 : 2) : 3;
+  static constexpr int NST = NCH < NMAX ? NCH : NMAX;
+  static constexpr int G = E == 4 ? MC : M % 4 == 0 ? 4 : 6;
+  static constexpr int SLOTS = M < NF * ND ? M : NF * ND;
+  // FP64: face table [f][p][q][NKP], phi'_k as int2, rows of an even number of entries; 2D: the reversed edge
+  // swaps the stored points, one order (NP = 1)
+  static constexpr int NP = D == 3 ? 6 : 1, NKP = (NK + 1) / 2 * 2;
+  static constexpr int PHI_BYTES = E == 8 ? NF * NP * NQ * NKP * 8 : 0;
+  static constexpr int STAGE = CPW * MC * NK * E;
+  static constexpr int HDR = CPW * NF * PDS * E, DELTA = SLOTS * 32 * E;
+  static constexpr int BARS = (1 + NST + 1) / 2 * 16;
+  static constexpr int WARP_BYTES = HDR + NST * STAGE + DELTA + BARS;
+  __host__ __device__ static constexpr int64_t index(int64_t cell, int m, int k) {  // of entry (m, k) of a cell in Pc
+    const int64_t t = cell / CPW;
+    return (((t * NCH + m / MC) * CPW + (cell - t * CPW)) * MC + m % MC) * NK + k;
+  }
+  static_assert(M % MC == 0 && MC % G == 0 && ND * KD <= PDS, "chunks of whole groups");
+  // blocks of 4 warps that shared memory lets an SM hold, and the register cap that goes with them
+  static constexpr int BLOCK_BYTES = PHI_BYTES + 16 + 4 * WARP_BYTES;
+  static constexpr int FIT = 227 * 1024 / (BLOCK_BYTES + 1024), BLOCKS = FIT < 4 ? FIT : 4;
+  static_assert((MC * NK * E) % 16 == 0 && (G * NK * E) % 16 == 0 && (PDS * E) % 16 == 0, "16-byte spans");
+};
+// Cells of Pc's allocation: whole tiles of 32 / (d + 2).
+inline int64_t tiled_cells(int d, int64_t n) {
+  const int64_t cpw = 32 / (d + 2);
+  return (n + cpw - 1) / cpw * cpw;
+}
+
+}  // namespace cteno
