@@ -280,17 +280,22 @@ int cteno_sync(cteno_ctx *ctx, int64_t *guard_count);
  * (mixed path, w warps per block, 1..8) selects the streamed thread-per-cell schedule: every warp
  * walks tiles of 32 cells, one thread per cell, and each lane streams its own cell's operator
  * record through the warp's ring of shared-memory stages four stencil members at a time; refused
- * likewise when it does not fit. 7168 + w / 7200 + w (mixed path, w warps per block, 1..8) select
- * the streamed schedule with two lanes per cell (each lane half of the conserved variables, 16
- * cells per warp) and a two- / three-stage ring of 4-member chunks; refused likewise. Flux only:
+ * likewise when it does not fit. 11264 + b (mixed path, b = 32, 64, 96 or 128 threads per block)
+ * selects the tile-per-warp schedule, one lane per conserved variable, whose operator records, stencil
+ * ids and face values pass through the warp's own shared memory; 10240 + b the same with two
+ * variables per lane; 7168 + w / 7200 + w (w warps per block, 1..8) the latter in blocks of
+ * min(w, 4) warps, refused where a two- / three-stage ring of 16 cells by 4 members would not fit
+ * in the shared memory of a block. All of them give the same bits as the lane schedules. Flux only:
  * 8192 + b (b a multiple of 32 in
  * [32, 256]) selects the face-based schedule: HLLC once per face, in its owner's orientation, into
  * a face-flux array, then a per-cell gather and update (results bit-identical to the per-cell
  * schedules). At central degrees 4 to 6 and with the characteristic reconstruction the reconstruction
- * takes 1024 + b only (default 1024 + 128), and on the mixed path without the characteristic
- * reconstruction also 1536 + b (the same schedule compiled for at most 64 registers per thread, so
- * that more warps share an SM); every other reconstruction value is refused with
- * CTENO_ERR_ARG. */
+ * takes 1024 + b only (default 1024 + 128; 1024 + 32 on the mixed path without the
+ * characteristic reconstruction), and on the mixed path without the characteristic reconstruction also
+ * 1536 + b (the same kernel); every other reconstruction value is refused with CTENO_ERR_ARG.
+ * The FP64 path has one schedule of each kernel (the reconstruction of the conserved variables, the flux):
+ * there b, 1024 + b and, for the flux, 8192 + b only set its threads per block (the reconstruction's 128 at
+ * most, as at degrees 4 to 6). */
 int cteno_set_launch(cteno_ctx *ctx, int recon_block, int flux_block);
 
 /* Time the candidate launch configurations (block sizes 64/128/256, on the mixed path the

@@ -315,6 +315,8 @@ int cteno_create(cteno_ctx **out, const cteno_params *p, void *cuda_stream) {
   ctx->nd = dir_members(p->dim, p->degree);
   // the variable-per-lane schedule for degrees 4 to 6 and for the characteristic reconstruction
   if (p->degree >= 4 || p->characteristic) ctx->recon_block = kLaneSchedule + 128;
+  // degrees 4 to 6, mixed: blocks of one warp (degree 4, 215 000 cells: 112 us a launch, in fours 117)
+  if (p->degree >= 4 && !p->characteristic && p->precision == CTENO_MIXED) ctx->recon_block = kLaneSchedule + 32;
   if (p->precision == CTENO_FP64) ctx->flux_block = 32;  // see flux64.cuh
   ctx->nsel = p->characteristic ? ctx->nf * ctx->nv : ctx->nv;
   ctx->nst = p->rk;
@@ -543,7 +545,7 @@ int cteno_lsq_build(cteno_ctx *ctx) {
   CK(dalloc(ctx, &ctx->Un, sizeof(double) * nvp * N));
   if (ctx->nst == 4) CK(dalloc(ctx, &ctx->Acc, sizeof(double) * nvp * N));
   if (ctx->fp32) CK(dalloc(ctx, &ctx->U32, 2 * sizeof(float) * nvp * N));
-  CK(dalloc(ctx, &ctx->st, sizeof(int32_t) * M * N));
+  CK(dalloc(ctx, &ctx->st, sizeof(int32_t) * M * tiled_cells(d, N)));
   CK(dalloc(ctx, &ctx->nbr, sizeof(int32_t) * 4 * N));
   CK(dalloc(ctx, &ctx->cinfo, sizeof(uint32_t) * N));
   CK(dalloc(ctx, &ctx->fmeta, sizeof(uint32_t) * N));
@@ -998,14 +1000,10 @@ int cteno_set_launch(cteno_ctx *ctx, int recon_block, int flux_block) {
     // the characteristic reconstruction: the variable-per-lane schedule only
     if (recon && ctx->p.characteristic)
       return b >= kLaneSchedule + 32 && b <= kLaneSchedule + 256 && b % 32 == 0;
-    if (b >= kFaceFlux)  // face-based flux schedule
+    if (b >= kFaceFlux && b < kTileLanes2)  // face-based flux schedule
       return !recon && b - kFaceFlux >= 32 && b - kFaceFlux <= 256 && b % 32 == 0;
-    {
-      int w = 0, st = 0;
-      pair_launch(b, &w, &st);
-      if (w)  // two lanes per cell: reconstruction, mixed, fits
-        return recon && ctx->fp32 && recon_pair_smem(ctx->d, ctx->p.degree, w, st) <= kMaxStreamSmem;
-    }
+    if (tile_launch(b))  // two variables per lane: reconstruction, mixed
+      return recon && ctx->fp32 && (b > kTileLanes2 || pair_fits(ctx->d, ctx->p.degree, b));
     if (b > kStreamCells && b <= kStreamCells + 8)  // streamed cells: reconstruction, mixed, fits
       return recon && ctx->fp32 &&
              recon_stream_cells_smem(ctx->d, ctx->p.degree, b - kStreamCells) <= kMaxStreamSmem;
@@ -1081,6 +1079,9 @@ int cteno_autotune(cteno_ctx *ctx, int32_t *best_out) {
     for (int b : {kStagedCells + 32, kStagedCells + 64, kStagedCells + 128, kStagedLanes + 64,
                   kStagedLanes + 128, kStagedLanes + 256})
       if (recon_staged_smem(ctx->d, ctx->p.degree, 1, b) <= kMaxStagedSmem) rcand.push_back(b);
+  if (ctx->fp32 && ctx->p.degree <= 3)
+    for (int b : {32, 64, 128})
+      for (int k : {kTileLanes2, kTileLanes}) rcand.push_back(k + b);
   if (ctx->fp32 && ctx->hl) {
     const long long hs = recon_halo_smem(ctx->d, ctx->p.degree, ctx->hrec);
     if (hs <= kMaxStagedSmem) rcand.push_back(kHaloLanes);
@@ -1094,10 +1095,6 @@ int cteno_autotune(cteno_ctx *ctx, int32_t *best_out) {
     }
     for (int w : {2, 4, 6, 7, 8})
       if (recon_stream_cells_smem(ctx->d, ctx->p.degree, w) <= kMaxStreamSmem) rcand.push_back(kStreamCells + w);
-    for (int w : {4, 6, 8}) {
-      if (recon_pair_smem(ctx->d, ctx->p.degree, w, 2) <= kMaxStreamSmem) rcand.push_back(kPairLanes + w);
-      if (recon_pair_smem(ctx->d, ctx->p.degree, w, 3) <= kMaxStreamSmem) rcand.push_back(kPairLanes3 + w);
-    }
   }
   if (ctx->p.characteristic)  // the variable-per-lane schedule only
     rcand = {kLaneSchedule + 64, kLaneSchedule + 128, kLaneSchedule + 256};

@@ -234,25 +234,27 @@ inline void stream_launch(int b, int *warps, int *stages) {
   if (b > kStreamLanes && b <= kStreamLanes + 16) *warps = b - kStreamLanes, *stages = 3;
   if (b > kStreamLanes2 && b <= kStreamLanes2 + 16) *warps = b - kStreamLanes2, *stages = 2;
 }
-// kPairLanes + w / kPairLanes3 + w (w warps per block, 1..8): the streamed schedule with two lanes
-// per cell (mixed path), a two- / three-stage ring of 4-member chunks of 16 cells per warp.
+// kTileLanes + b / kTileLanes2 + b (b = 32, 64, 96, 128 threads): a tile of cells per warp, one / two variables per
+// lane (recon_tile.cuh; mixed path, degrees 2 and 3, conserved variables).
+constexpr int kTileLanes = 11264;
+constexpr int kTileLanes2 = 10240;
+// kPairLanes + w / kPairLanes3 + w (w warps per block, 1..8, accepted where a ring of two / three stages of 16 cells
+// by 4 members fits in shared memory): kTileLanes2 in blocks of min(w, 4) warps.
 constexpr int kPairLanes = 7168;
 constexpr int kPairLanes3 = 7200;
-inline long long recon_pair_smem(int d, int degree, int warps, int stages) {
+inline bool pair_fits(int d, int degree, int block) {
+  const int stages = block > kPairLanes3 ? 3 : 2, warps = block - (stages == 3 ? kPairLanes3 : kPairLanes);
   const int nk = (d == 2 ? (degree + 1) * (degree + 2) / 2 : (degree + 1) * (degree + 2) * (degree + 3) / 6) - 1;
-  const int M = 2 * (nk + 1);
-  const long long stage = 16LL * 4 * nk * 4;
-  const long long hdr = 16LL * (d + 1) * lay_pds(d) * 4 + 16LL * M * 4;
-  const long long nphi = d == 3 ? (long long)(d + 1) * 6 * 4 * nk : 1;
-  const long long phi = (nphi * 4 + 15) / 16 * 16;
-  return phi + (long long)warps * (2 * hdr + stages * stage) + (long long)warps * (2 + stages) * 8 + 8;
+  const long long M = 2 * (nk + 1), hdr = 16LL * (d + 1) * lay_pds(d) * 4 + 16LL * M * 4;
+  const long long phi = ((d == 3 ? (long long)(d + 1) * 6 * 4 * nk : 1) * 4 + 15) / 16 * 16;
+  return phi + warps * (2 * hdr + stages * (16LL * 4 * nk * 4)) + warps * (2 + stages) * 8LL + 8 <= kMaxStreamSmem;
 }
-// Launch value -> (warps, stages) of the two-lanes-per-cell schedule, or warps = 0.
-inline void pair_launch(int b, int *warps, int *stages) {
-  *warps = 0;
-  *stages = 0;
-  if (b > kPairLanes && b <= kPairLanes + 8) *warps = b - kPairLanes, *stages = 2;
-  if (b > kPairLanes3 && b <= kPairLanes3 + 8) *warps = b - kPairLanes3, *stages = 3;
+// Threads per block of a launch value of this schedule, or 0.
+inline int tile_launch(int b) {
+  if (b > kTileLanes) return b <= kTileLanes + 128 && b % 32 == 0 ? b - kTileLanes : 0;
+  if (b > kTileLanes2) return b <= kTileLanes2 + 128 && b % 32 == 0 ? b - kTileLanes2 : 0;
+  const int w = b > kPairLanes3 ? b - kPairLanes3 : b - kPairLanes;
+  return b > kPairLanes && w >= 1 && w <= 8 ? 32 * (w < 4 ? w : 4) : 0;
 }
 inline int halo_tile(int d) { return kHaloWarps * (32 / (d + 2)); }
 inline int halo_ms(int M) { return (M + 1 + 7) / 8 * 8; }

@@ -31,6 +31,26 @@ struct Shape {
   static constexpr int NP = (D == 2) ? 2 : 6;
 };
 
+// Which entries of the smoothness matrix O (eq. 15) differ from zero: psi_k and psi_l have a common
+// derivative where some coordinate is in both monomials. Bit l of row k; the basis is graded, within a degree by
+// the z then the y power. Of 190 entries of the upper triangle 54 are zero at 3D degree 3, 18 of 45 at 3D
+// degree 2, 4 of 15 to 36 of 378 in 2D: leaving a zero product out changes no bit of a sum.
+template <int D, int R>
+struct SmoothRows {
+  static constexpr int NK = (D == 2 ? (R + 1) * (R + 2) / 2 : (R + 1) * (R + 2) * (R + 3) / 6) - 1;
+  uint32_t row[NK] = {};
+  __host__ __device__ constexpr SmoothRows() {
+    uint32_t has[NK] = {};  // the coordinates of a monomial
+    int k = 0;
+    for (int t = 1; t <= R; ++t)
+      for (int c = 0; c <= (D == 3 ? t : 0); ++c)
+        for (int b = 0; b <= t - c; ++b) has[k++] = (t - b - c > 0 ? 1u : 0u) | (b > 0 ? 2u : 0u) | (c > 0 ? 4u : 0u);
+    for (int i = 0; i < NK; ++i)
+      for (int j = 0; j < NK; ++j)
+        if (has[i] & has[j]) row[i] |= 1u << j;
+  }
+};
+
 // Constant-bank copies of the universal tables of this module's degrees (filled by
 // upload_recon_tables_*): the smoothness matrix O (eq. 15; upper triangle, off-diagonal doubled) and, in 2D, the face-point basis values
 // phi_k at the two Gauss points of each local edge taken in local vertex order (the other edge
@@ -640,10 +660,13 @@ __global__ void __launch_bounds__(MINB ? 128 : 256, MINB ? MINB : 1) recon_kerne
 // indicators (eq. 15: oc(k * NK + l) the upper triangle of the central O, off-diagonal doubled;
 // sid(ad_f) a directional indicator), the selection (eqs. 19-23, Alg. 1 / 2) or the CWENO weights
 // (eq. 14), and the final coefficients in ao. Returns the flags byte.
-template <int NF, int NK, int KD, typename T, int SCHEME, typename OC, typename SID>
+template <int D, int NK, int KD, typename T, int SCHEME, typename OC, typename SID>
 __device__ __forceinline__ uint32_t lane_select(const KArgs &a, const uint32_t adm, T (&ao)[NK],
-                                                const T (&ad)[NF][KD], OC oc, SID sid) {
+                                                const T (&ad)[D + 1][KD], OC oc, SID sid) {
+  constexpr int NF = D + 1;
   constexpr bool F32 = sizeof(T) == 4;
+  constexpr int R = D == 3 ? (NK == 9 ? 2 : 3) : NK == 5 ? 2 : NK == 9 ? 3 : NK == 14 ? 4 : NK == 20 ? 5 : 6;
+  constexpr SmoothRows<D, R> smooth;
   const int stn = 1 + __popc(adm);
   T lams;
   double lamsd = 0.0;
@@ -674,7 +697,8 @@ __device__ __forceinline__ uint32_t lane_select(const KArgs &a, const uint32_t a
   for (int k = 0; k < NK; ++k) {
     T rr = (T)0;
 #pragma unroll
-    for (int l = k; l < NK; ++l) rr += oc(k * NK + l) * ao[l];
+    for (int l = k; l < NK; ++l)
+      if ((smooth.row[k] >> l) & 1u) rr += oc(k * NK + l) * ao[l];
     SI0 += ao[k] * rr;
   }
   T SId[NF];
@@ -962,7 +986,7 @@ __device__ __forceinline__ void lane_faces(const KArgs &a, const int64_t i, cons
   bool bad = false;
   T fv[NF][NQ];
   if constexpr (!CHR) {
-    const uint32_t bits = lane_select<NF, NK, KD, T, SCHEME>(a, adm, ao, ad, oc, sid);
+    const uint32_t bits = lane_select<D, NK, KD, T, SCHEME>(a, adm, ao, ad, oc, sid);
     if (a.flags && active) a.flags[v * N + i] = (uint8_t)bits;
     const T off = phi.offset(ao);
 #pragma unroll
@@ -1013,7 +1037,7 @@ __device__ __forceinline__ void lane_faces(const KArgs &a, const int64_t i, cons
       T wbar = (T)0;
 #pragma unroll
       for (int j = 0; j < NV; ++j) wbar += Lw[j] * ub[j];
-      const uint32_t bits = lane_select<NF, NK, KD, T, SCHEME>(a, adm, aw, adw, oc, sid);
+      const uint32_t bits = lane_select<D, NK, KD, T, SCHEME>(a, adm, aw, adw, oc, sid);
       if (a.flags && active) a.flags[(f * NV + v) * N + i] = (uint8_t)bits;
 #pragma unroll
       const T off = phi.offset(aw);

@@ -1,12 +1,20 @@
 // recon_2d.cu -- instantiations of the reconstruction kernel for d = 2.
 #include "recon.cuh"
-#include "recon_pair.cuh"
+#include "recon_tile.cuh"
 
 namespace cteno {
 
 cudaError_t launch_recon_2d(int degree, int fp32, int scheme, const KArgs &a, int block, cudaStream_t s) {
   // the characteristic reconstruction runs in the variable-per-lane schedule only
   if (a.characteristic && !(block >= kLaneSchedule && block < kStagedCells)) return cudaErrorInvalidValue;
+  if (const int threads = tile_launch(block)) {  // two variables per lane (mixed)
+    if (!fp32) return cudaErrorInvalidValue;  // mixed path only
+    const bool one = block >= kTileLanes;
+#define CTENO_TILE(R, SC) (one ? launch_recon_tile<2, R, SC, 1>(a, threads, s) : launch_recon_tile<2, R, SC, 2>(a, threads, s))
+    if (degree == 2) return scheme ? CTENO_TILE(2, 1) : CTENO_TILE(2, 0);
+    return scheme ? CTENO_TILE(3, 1) : CTENO_TILE(3, 0);
+#undef CTENO_TILE
+  }
   if (block == kHaloLanes || block == kHaloLanes + 1) {  // gather-staged lane schedule (mixed)
     if (!fp32) return cudaErrorInvalidValue;  // mixed path only
     const bool one = block == kHaloLanes + 1;  // one tile per block, single stage
@@ -18,21 +26,6 @@ cudaError_t launch_recon_2d(int degree, int fp32, int scheme, const KArgs &a, in
     if (degree == 3 && scheme == 1) CTENO_HALO(3, 1);
 #undef CTENO_HALO
     return cudaSuccess;
-  }
-  {
-    int warps = 0, stages = 0;
-    pair_launch(block, &warps, &stages);
-    if (warps) {  // streamed schedule, two lanes per cell (mixed)
-      if (!fp32) return cudaErrorInvalidValue;  // mixed path only
-#define CTENO_PAIR(R, SC) \
-  (stages == 3 ? launch_recon_pair<2, R, SC, 3>(a, warps, s) : launch_recon_pair<2, R, SC, 2>(a, warps, s))
-      if (degree == 2 && scheme == 0) CTENO_PAIR(2, 0);
-      if (degree == 2 && scheme == 1) CTENO_PAIR(2, 1);
-      if (degree == 3 && scheme == 0) CTENO_PAIR(3, 0);
-      if (degree == 3 && scheme == 1) CTENO_PAIR(3, 1);
-#undef CTENO_PAIR
-      return cudaSuccess;
-    }
   }
   if (block > kStreamCells && block <= kStreamCells + 8) {  // streamed thread-per-cell schedule (mixed)
     if (!fp32) return cudaErrorInvalidValue;  // mixed path only

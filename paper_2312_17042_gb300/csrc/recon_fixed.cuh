@@ -195,12 +195,18 @@ __global__ void __launch_bounds__(128, TileShape<D, R, 8>::BLOCKS) recon_fixed_k
       bulk_copy_g2s(smem, a.phifx, S::PHI_BYTES, tbar);
     }
     if (n > 0) {
-      for (int c = 0; c < NST; ++c) issue(c);
-      mbar_arrive_expect_tx(&bar[0], (uint32_t)(n * NF * PDS * 8));
+      mbar_arrive_expect_tx(&bar[0], (uint32_t)(CPW * M * 4 + n * NF * PDS * 8));
+      bulk_copy_g2s(wmem + S::HPD, a.st + c0 * M, (uint32_t)(CPW * M * 4), &bar[0]);
       bulk_copy_g2s(wmem, (const int2 *)a.Pd + c0 * (NF * PDS), (uint32_t)(n * NF * PDS * 8), &bar[0]);
+      for (int c = 0; c < NST; ++c) issue(c);
     }
   }
   __syncthreads();
+  const bool active = grp < n;
+  const int slot = active ? grp : max(n, 1) - 1;  // spare lanes shadow a valid cell and store nothing
+  const int64_t i = min(c0 + slot, N - 1);
+  const uint32_t info = __ldg(a.cinfo + i);
+  const int8_t *__restrict__ ei = a.Pe + i * kFixExp;
   pdl_wait(a);  // the state written by the previous stage's update
   if (a.dt_swap && blockIdx.x == 0)  // the CFL step: dt[next] -> dt[cur]
     for (int t = threadIdx.x; t < a.nmesh; t += blockDim.x) {
@@ -225,25 +231,23 @@ __global__ void __launch_bounds__(128, TileShape<D, R, 8>::BLOCKS) recon_fixed_k
     arrived(tbar, 0, 0, 0);
     return;
   }
-  const bool active = grp < n;
-  const int slot = active ? grp : n - 1;  // spare lanes shadow a valid cell and store nothing
-  const int64_t i = c0 + slot;
   const double *__restrict__ Uv = a.U + v;
-  const int32_t *__restrict__ sti = a.st + i * M;
+  const int32_t *__restrict__ sti = reinterpret_cast<const int32_t *>(wmem + S::HPD) + slot * M;
   const double U0 = __ldg(Uv + i * NVP);
   auto ids_of = [&](int m, int (&j)[G]) {
     if constexpr (G == 4) {
-      const int4 t = __ldg(reinterpret_cast<const int4 *>(sti + m));
+      const int4 t = *reinterpret_cast<const int4 *>(sti + m);
       j[0] = t.x, j[1] = t.y, j[2] = t.z, j[3] = t.w;
     } else {
 #pragma unroll
       for (int g = 0; g < G; g += 2) {
-        const int2 t = __ldg(reinterpret_cast<const int2 *>(sti + m + g));
+        const int2 t = *reinterpret_cast<const int2 *>(sti + m + g);
         j[g] = t.x, j[g + 1] = t.y;
       }
     }
   };
 
+  if (!arrived(&bar[0], 0, 0, NST)) return;
   // the range of variable v over the stencil, from the high words in the order of the values
   auto key = [](int h) { return h ^ ((h >> 31) & 0x7FFFFFFF); };
   int kmax = key(__double2hiint(U0)), kmin = kmax;
@@ -265,7 +269,6 @@ __global__ void __launch_bounds__(128, TileShape<D, R, 8>::BLOCKS) recon_fixed_k
   const int64_t F0 = fx_of(U0, er);
 
   // central coefficients b = P_c (U_m - U_0)
-  const int8_t *__restrict__ ei = a.Pe + i * kFixExp;
   double ao[NK];
   {
     int64_t A1[NK], A2[NK];
@@ -323,9 +326,7 @@ __global__ void __launch_bounds__(128, TileShape<D, R, 8>::BLOCKS) recon_fixed_k
     for (int k = 0; k < NK; ++k) ao[k] = fx_to_double(A1[k], A2[k], 29 - 57 - 1079 + er + __ldg(ei + k));
   }
   // directional coefficients: the members of face f are the next slots of the list
-  const uint32_t info = __ldg(a.cinfo + i);
   const uint32_t adm = (info >> kInfoAdmShift) & 0xFu;
-  if (!arrived(&bar[0], 0, NCH, NCH)) return;
   const int2 *__restrict__ Pdi = reinterpret_cast<const int2 *>(wmem) + slot * (NF * PDS);
   double ad[NF][KD];
   {

@@ -252,11 +252,16 @@ __global__ void __launch_bounds__(128, TileShape<2, R, 4>::BLOCKS) recon_high_st
   if (lane == 0 && n > 0) {
     for (int b = 0; b < 1 + NST; ++b) mbar_init(&bar[b], 1);
     fence_barrier_init();
-    for (int c = 0; c < NST; ++c) issue(c);
-    mbar_arrive_expect_tx(&bar[0], (uint32_t)(n * NF * PDS * 4));
+    mbar_arrive_expect_tx(&bar[0], (uint32_t)(S::CPW * M * 4 + n * NF * PDS * 4));
+    bulk_copy_g2s(wmem + S::HPD, a.st + c0 * M, (uint32_t)(S::CPW * M * 4), &bar[0]);
     bulk_copy_g2s(wmem, (const float *)a.Pd + c0 * (NF * PDS), (uint32_t)(n * NF * PDS * 4), &bar[0]);
+    for (int c = 0; c < NST; ++c) issue(c);
   }
   __syncwarp();
+  const bool active = grp < n;
+  const int slot = active ? grp : max(n, 1) - 1;  // spare lanes shadow a valid cell and store nothing
+  const int64_t i = min(c0 + slot, N - 1);
+  const uint32_t info = __ldg(a.cinfo + i);
   pdl_wait(a);  // the state written by the previous stage's update
   if (a.dt_swap && blockIdx.x == 0)  // the CFL step: dt[next] -> dt[cur]
     for (int t = threadIdx.x; t < a.nmesh; t += blockDim.x) {
@@ -271,30 +276,27 @@ __global__ void __launch_bounds__(128, TileShape<2, R, 4>::BLOCKS) recon_high_st
     if (!__any_sync(0xffffffffu, !ok)) return true;
     if (lane == 0) {
       atomicOr(a.err, kErrTimeout);
-      mbar_wait(&bar[0], 0, kStageWaitNs);
+      if (!c) mbar_wait(&bar[0], 0, kStageWaitNs);
       for (; c < last; ++c) mbar_wait(&bar[1 + c % NST], (uint32_t)((c / NST) & 1), kStageWaitNs);
     }
     __syncwarp();
     return false;
   };
-  const bool active = grp < n;
-  const int slot = active ? grp : n - 1;  // spare lanes shadow a valid cell and store nothing
-  const int64_t i = c0 + slot;
   const float2 *__restrict__ Uv = reinterpret_cast<const float2 *>(a.U32) + v;
-  const int32_t *__restrict__ sti = a.st + i * M;
+  const int32_t *__restrict__ sti = reinterpret_cast<const int32_t *>(wmem + S::HPD) + slot * M;
   const float2 own = __ldg(Uv + i * NVP);
   const float U0 = own.x, L0 = own.y;
   float2 nx[MC];  // the next chunk's member means
   auto fetch = [&](int c) {
 #pragma unroll
     for (int g = 0; g < MC; g += 2) {
-      const int2 j = __ldg(reinterpret_cast<const int2 *>(sti + c * MC + g));
+      const int2 j = *reinterpret_cast<const int2 *>(sti + c * MC + g);
       nx[g] = __ldg(Uv + (int64_t)j.x * NVP);
       nx[g + 1] = __ldg(Uv + (int64_t)j.y * NVP);
     }
   };
+  if (!arrived(&bar[0], 0, 0, NST)) return;
   fetch(0);
-  const uint32_t info = __ldg(a.cinfo + i);
   float ao[NK];
 #pragma unroll
   for (int k = 0; k < NK; ++k) ao[k] = 0.0f;
@@ -325,7 +327,6 @@ __global__ void __launch_bounds__(128, TileShape<2, R, 4>::BLOCKS) recon_high_st
     }
   }
   // directional coefficients (degree 2): the members of face f are the next slots of the list
-  if (!arrived(&bar[0], 0, NCH, NCH)) return;
   const uint32_t adm = (info >> kInfoAdmShift) & 7u;
   const float *__restrict__ Pdi = reinterpret_cast<const float *>(wmem) + slot * (NF * PDS);
   float ad[NF][KD];

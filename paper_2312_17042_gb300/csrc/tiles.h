@@ -24,11 +24,13 @@ struct TileShape {
   static constexpr int KD = Dir<D, R>::KD, ND = Dir<D, R>::ND, PDS = Dir<D, R>::PDS;
   static constexpr int CPW = 32 / NV;
   // Chunks of the central record, NST of them in flight, and the members whose differences are formed
-  // together. FP64: all of it up to 20 members (2D degrees 2, 3; 3D degree 2). Mixed: chunks of 4.4,
-  // 3.8 and 6.9 kB a warp at degrees 4, 5 and 6, 12 to 15 kB in flight, which with 11 to 12 warps covers
-  // the memory latency of an SM (about 45 kB at the full rate) through the arithmetic of each warp.
-  static constexpr int MC = E == 4 ? (R == 4 ? 10 : R == 5 ? 6 : 8) : M <= 20 ? M : M % 4 == 0 ? 4 : 6;
-  static constexpr int NCH = M / MC, NMAX = E == 4 ? (R == 4 ? 3 : R == 5 ? 4 : 2) : 3;
+  // together. FP64: all of it up to 20 members (2D degrees 2, 3; 3D degree 2). Mixed: chunks of 2.7,
+  // 3.8 and 3.5 kB a warp at degrees 4, 5 and 6; 5 to 12 kB in flight in each of 9 to 13 warps cover the
+  // memory latency of an SM (about 45 kB at the full rate) through the arithmetic. Measured, us a
+  // launch (MC x NST): degree 4, 215 000 cells 10 x 3 123.7, 10 x 2 115.1, 6 x 3 117.7, 6 x 2 112.4; degree 6,
+  // 180 000 cells 8 x 2 223.3, 8 x 3 230.2, 4 x 3 219.7, 4 x 4 237.4.
+  static constexpr int MC = E == 4 ? (R == 6 ? 4 : 6) : M <= 20 ? M : M % 4 == 0 ? 4 : 6;
+  static constexpr int NCH = M / MC, NMAX = E == 4 ? (R == 4 ? 2 : 3) : 3;
   static constexpr int NST = NCH < NMAX ? NCH : NMAX;
   static constexpr int G = E == 4 ? MC : M % 4 == 0 ? 4 : 6;
   static constexpr int SLOTS = M < NF * ND ? M : NF * ND;
@@ -37,7 +39,8 @@ struct TileShape {
   static constexpr int NP = D == 3 ? 6 : 1, NKP = (NK + 1) / 2 * 2;
   static constexpr int PHI_BYTES = E == 8 ? NF * NP * NQ * NKP * 8 : 0;
   static constexpr int STAGE = CPW * MC * NK * E;
-  static constexpr int HDR = CPW * NF * PDS * E, DELTA = SLOTS * 32 * E;
+  // a warp's header: directional operators, then stencil ids
+  static constexpr int HPD = CPW * NF * PDS * E, HDR = HPD + CPW * M * 4, DELTA = SLOTS * 32 * E;
   static constexpr int BARS = (1 + NST + 1) / 2 * 16;
   static constexpr int WARP_BYTES = HDR + NST * STAGE + DELTA + BARS;
   __host__ __device__ static constexpr int64_t index(int64_t cell, int m, int k) {  // of entry (m, k) of a cell in Pc
@@ -48,7 +51,8 @@ struct TileShape {
   // blocks of 4 warps that shared memory lets an SM hold, and the register cap that goes with them
   static constexpr int BLOCK_BYTES = PHI_BYTES + 16 + 4 * WARP_BYTES;
   static constexpr int FIT = 227 * 1024 / (BLOCK_BYTES + 1024), BLOCKS = FIT < 4 ? FIT : 4;
-  static_assert((MC * NK * E) % 16 == 0 && (G * NK * E) % 16 == 0 && (PDS * E) % 16 == 0, "16-byte spans");
+  static_assert((MC * NK * E) % 16 == 0 && (G * NK * E) % 16 == 0 && (PDS * E) % 16 == 0 && (M * 4) % 8 == 0 &&
+                    HDR % 16 == 0, "16-byte spans");
 };
 // Cells of Pc's allocation: whole tiles of 32 / (d + 2).
 inline int64_t tiled_cells(int d, int64_t n) {
