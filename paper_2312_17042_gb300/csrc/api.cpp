@@ -317,6 +317,13 @@ int cteno_create(cteno_ctx **out, const cteno_params *p, void *cuda_stream) {
   if (p->degree >= 4 || p->characteristic) ctx->recon_block = kLaneSchedule + 128;
   // degrees 4 to 6, mixed: blocks of one warp (degree 4, 215 000 cells: 112 us a launch, in fours 117)
   if (p->degree >= 4 && !p->characteristic && p->precision == CTENO_MIXED) ctx->recon_block = kLaneSchedule + 32;
+  // mixed, 2D degrees 2 and 3: a tile per warp and the register-capped flux; elsewhere the face-based flux. 131 072
+  // triangles: 19.9 + 16.3 us a launch against 30.8 + 20.4 with a thread per cell; the face-based flux takes 16.7
+  // us there, and 26 against 36 us at 215 000 cells of degree 4, 104 against 193 us at 663 552 tetrahedra. (The 3D
+  // reconstruction stays with a thread per cell, whose face values are rounded differently: cteno_autotune.)
+  if (p->precision == CTENO_MIXED) ctx->flux_block = p->dim == 2 && p->degree <= 3 ? -128 : kFaceFlux + 128;
+  if (p->precision == CTENO_MIXED && p->dim == 2 && p->degree <= 3 && !p->characteristic)
+    ctx->recon_block = kTileLanes + 32;
   if (p->precision == CTENO_FP64) ctx->flux_block = 32;  // see flux64.cuh
   ctx->nsel = p->characteristic ? ctx->nf * ctx->nv : ctx->nv;
   ctx->nst = p->rk;
