@@ -26,9 +26,11 @@
 // differences of the directional members (the first slots of the stencil list) wait in shared
 // memory between the two products.
 //
-// Measured per launch against the FP64 schedules it replaced (bound by the FP64 pipe, 61 to 86 %
-// of its rate): 2D degree 3, 131 072 cells 534 -> 126 us; 3D degree 3, 24 576 cells 432 -> 142 us;
-// 2D degree 5, 4200 cells 81 -> 37 us; 2D degree 2, 2048 cells 19 (51 in blocks of 128) -> 13 us.
+// Measured per launch against the FP64 schedules it replaced (bound by the FP64 pipe, 61 to 86 % of its
+// rate): 2D degree 3, 131 072 cells 534 -> 110 us; 3D degree 3, 24 576 cells 432 (553 in blocks of 128) -> 127
+// us; 2D degree 5, 4200 cells 81 -> 35 us; 2D degree 2, 2048 cells 19 (51 in blocks of 128) -> 12 us. It is
+// now bound by the integer pipe (shifts and 64-bit sums of the conversions, 63 % busy at 2D degree 3), the
+// small meshes by the length of a warp's chain.
 #pragma once
 
 #include "recon.cuh"
@@ -41,43 +43,36 @@ namespace cteno {
 __device__ __forceinline__ void fx_mac(int64_t &acc, const int a, const int b) {
   asm("mad.wide.s32 %0, %1, %2, %0;" : "+l"(acc) : "r"(a), "r"(b));
 }
-// x = h 2^29 + l, |l| <= 2^28.
-__device__ __forceinline__ int2 fx_split(const int64_t x) {
-  const int64_t t = x + (1 << 28);
+// x = h 2^29 + l, |l| <= 2^28, from x + 2^28.
+__device__ __forceinline__ int2 fx_split(const int64_t t) {
   return make_int2((int)(t >> 29), (int)((uint32_t)t & 0x1FFFFFFFu) - (1 << 28));
 }
 
-// u in units of 2^(e - 1079), e the biased exponent of the unit's block, modulo 2^64 (a value far
-// below the unit gives 0; e >= 64, so zeros and subnormals do).
-__device__ __forceinline__ int64_t fx_of(const double u, const int e) {
-  const int hi = __double2hiint(u);
-  const uint64_t m = ((uint64_t)((hi & 0xFFFFF) | 0x100000) << 32) | (uint32_t)__double2loint(u);
-  const int s = ((hi >> 20) & 0x7FF) - e + 4;
-  uint64_t f;
-  asm("shl.b64 %0, %1, %2;" : "=l"(f) : "l"(m), "r"(max(s, 0)));
-  asm("shr.u64 %0, %1, %2;" : "=l"(f) : "l"(f), "r"(max(-s, 0)));
+// u in units of 2^(e - 1079) less `base`, e the biased exponent of the unit's block: |u| < 2^(e - 1015), modulo
+// 2^64, truncated (a value far below the unit gives 0; e >= 64, so zeros and subnormals do).
+__device__ __forceinline__ int64_t fx_of(const double u, const int e, const int64_t base) {
+  const int hi = __double2hiint(u), lo = __double2loint(u);
+  const uint64_t m = ((uint64_t)(__funnelshift_l(lo, hi, 11) | 0x80000000u) << 32) | ((uint32_t)lo << 11);
+  uint64_t f;  // the shift is 7 to 64 and more places for |u| < 2^(e - 1022), 0 at the limit above
+  asm("shr.u64 %0, %1, %2;" : "=l"(f) : "l"(m), "r"(7 + e - ((hi >> 20) & 0x7FF)));
   const int64_t sg = hi >> 31;
-  return (int64_t)(f ^ (uint64_t)sg) - sg;
+  return (int64_t)(f ^ (uint64_t)sg) - sg - base;
 }
 
-// (A1 2^29 + A2) 2^x rounded to FP64 (magnitudes one unit of the last place of A2 off when negative).
+// (A1 2^29 + A2) 2^x rounded to FP64, from its integer part in units of 2^(x + 29) (what lies below is less
+// than the last places of the factors' integers); 0 outside the normal numbers.
 __device__ __forceinline__ double fx_to_double(int64_t A1, const int64_t A2, const int x) {
   A1 += A2 >> 29;
   const uint32_t sg = (uint32_t)(A1 >> 63);
-  uint32_t w2 = (uint32_t)(A1 >> 32) ^ sg, w1 = (uint32_t)A1 ^ sg, w0 = ((uint32_t)A2 << 3) ^ sg;
-  int e = 95 - 3 + 1022 + x;  // biased exponent less one of a leading bit 31 of w2
-  if (w2 == 0u) {
-    w2 = w1, w1 = w0, w0 = 0u, e -= 32;
-    if (w2 == 0u) w2 = w1, w1 = 0u, e -= 32;
-  }
-  const int c = __clz((int)w2);
-  const uint32_t mh = __funnelshift_l(w1, w2, c), ml = __funnelshift_l(w0, w1, c);
+  uint32_t w1 = (uint32_t)(A1 >> 32) ^ sg, w0 = (uint32_t)A1 ^ sg;  // the magnitude, less one unit when negative
+  int e = 63 + 29 + 1022 + x;  // biased exponent less one of a leading bit 31 of w1
+  if (w1 == 0u) w1 = w0, w0 = 0u, e -= 32;
+  const int c = __clz((int)w1);
+  const uint32_t mh = __funnelshift_l(w0, w1, c), ml = w0 << (c & 31);
   e -= c;
-  const uint64_t m = (((uint64_t)mh << 32) | ml) >> 11;
-  uint64_t b = m + ((ml >> 10) & 1u) + ((uint64_t)(uint32_t)e << 52);
-  if (e < 0 || mh == 0u) b = 0;             // zero, or below the normal numbers
-  if (e > 2045) b = 0x7FF0000000000000ull;
-  return __longlong_as_double((long long)(b | ((uint64_t)(sg & 0x80000000u) << 32)));
+  const uint64_t b = ((((uint64_t)mh << 32) | ml) >> 11) + ((ml >> 10) & 1u) + ((uint64_t)(uint32_t)e << 52);
+  const bool ok = (uint32_t)e <= 2045u && mh != 0u;
+  return __hiloint2double(ok ? (int)((uint32_t)(b >> 32) | (sg & 0x80000000u)) : 0, ok ? (int)(uint32_t)b : 0);
 }
 
 // x truncated to FP32, 0 below its normal range, infinite above it (and for non-finite x).
@@ -190,7 +185,7 @@ __global__ void __launch_bounds__(128, TileShape<D, R, 8>::BLOCKS) recon_fixed_k
     for (int b = 0; b < 1 + NST; ++b) mbar_init(&bar[b], 1);
     if (threadIdx.x == 0) mbar_init(tbar, 1);
     fence_barrier_init();
-    if (threadIdx.x == 0) {
+    if (S::PHI_BYTES && threadIdx.x == 0) {
       mbar_arrive_expect_tx(tbar, S::PHI_BYTES);
       bulk_copy_g2s(smem, a.phifx, S::PHI_BYTES, tbar);
     }
@@ -220,7 +215,7 @@ __global__ void __launch_bounds__(128, TileShape<D, R, 8>::BLOCKS) recon_fixed_k
     if (!__any_sync(0xffffffffu, !ok)) return true;
     if (lane == 0) {
       atomicOr(a.err, kErrTimeout);
-      mbar_wait(tbar, 0, kStageWaitNs);
+      if (S::PHI_BYTES) mbar_wait(tbar, 0, kStageWaitNs);
       if (n > 0) mbar_wait(&bar[0], 0, kStageWaitNs);
       for (; n > 0 && c < last; ++c) mbar_wait(&bar[1 + c % NST], (uint32_t)((c / NST) & 1), kStageWaitNs);
     }
@@ -228,7 +223,7 @@ __global__ void __launch_bounds__(128, TileShape<D, R, 8>::BLOCKS) recon_fixed_k
     return false;
   };
   if (n == 0) {  // a warp past the last cell; the block's copy may be its own
-    arrived(tbar, 0, 0, 0);
+    if (S::PHI_BYTES) arrived(tbar, 0, 0, 0);
     return;
   }
   const double *__restrict__ Uv = a.U + v;
@@ -263,10 +258,12 @@ __global__ void __launch_bounds__(128, TileShape<D, R, 8>::BLOCKS) recon_fixed_k
     }
   }
   const double range = __hiloint2double(key(kmax), kmax < 0 ? 0 : -1) - __hiloint2double(key(kmin), kmin < 0 ? -1 : 0);
-  const int er = max((__double2hiint(range) >> 20) & 0x7FF, 64);  // |U_m - U_0| < 2^(er - 1022)
+  // |U_m - U_0| < 2^(er - 1022); the unit 2^(er - 1079) at least 2^-64 of the largest |U_m|
+  const int eu = (max(kmax, ~kmin) >> 20) & 0x7FF;
+  const int er = max((__double2hiint(range) >> 20) & 0x7FF, max(eu - 7, 64));
   // a non-finite member makes every coefficient NaN
   const bool finite = kmax < 0x7FF00000 && kmin > (int)0x800FFFFF && er < 0x7FF;
-  const int64_t F0 = fx_of(U0, er);
+  const int64_t F0 = fx_of(U0, er, 1 << 28);
 
   // central coefficients b = P_c (U_m - U_0)
   double ao[NK];
@@ -288,7 +285,7 @@ __global__ void __launch_bounds__(128, TileShape<D, R, 8>::BLOCKS) recon_fixed_k
       int2 dx[G];
 #pragma unroll
       for (int g = 0; g < G; ++g) {
-        dx[g] = fx_split(fx_of(un[g], er) - F0);
+        dx[g] = fx_split(fx_of(un[g], er, F0));
         if (m + g < SLOTS) sdel[(m + g) * 32] = dx[g];
       }
       if (m + G < M) {
@@ -462,19 +459,20 @@ __global__ void __launch_bounds__(128, TileShape<D, R, 8>::BLOCKS) recon_fixed_k
 #pragma unroll
   for (int k = 0; k < NK; ++k) {
     nan = nan || ((__double2hiint(ao[k]) >> 20) & 0x7FF) == 0x7FF;
-    bx[k] = fx_split(fx_of(ao[k], ef - a.phi_exp[k]));
+    bx[k] = fx_split(fx_of(ao[k], ef - a.phi_exp[k], -(1 << 28)));
   }
   const uint32_t perm = info >> kInfoPermShift;
   double *__restrict__ Ufi = (double *)a.Uf + i * (int64_t)(NF * NQ * NV) + v;
   auto slot_of = [&](int f, int q) {  // 2D: edge points in sorted-vertex order
     return (f * NQ + ((D == 2 && ((perm >> (3 * f)) & 7u)) ? NQ - 1 - q : q)) * NV;
   };
-  bool doubt = false;
-  if (!arrived(tbar, 0, NCH, NCH)) return;
+  float low = INFINITY;  // bounds of the face values in FP32: the smallest, the bits of the largest magnitude
+  uint32_t top = 0u;
+  if (S::PHI_BYTES && !arrived(tbar, 0, NCH, NCH)) return;
 #pragma unroll 1  // straight-line code for every face would not fit the instruction cache
   for (int f = 0; f < NF; ++f) {
     const int p = D == 3 ? (perm >> (3 * f)) & 7u : 0;
-    const int4 *__restrict__ ph = sPhi + (f * NP + p) * (NQ * NKP / 2);
+    const int4 *__restrict__ ph = (S::PHI_BYTES ? sPhi : reinterpret_cast<const int4 *>(a.phifx)) + (f * NP + p) * (NQ * NKP / 2);
     int64_t A1[NQ], A2[NQ];
 #pragma unroll
     for (int q = 0; q < NQ; ++q) A1[q] = A2[q] = 0;
@@ -482,7 +480,9 @@ __global__ void __launch_bounds__(128, TileShape<D, R, 8>::BLOCKS) recon_fixed_k
     for (int k = 0; k < NK; k += 2)
 #pragma unroll
       for (int q = 0; q < NQ; ++q) {
-        const int4 x = ph[(q * NKP + k) / 2];
+        int4 x;
+        if constexpr (S::PHI_BYTES > 0) x = ph[(q * NKP + k) / 2];
+        else x = __ldg(ph + (q * NKP + k) / 2);
         fx_mac(A1[q], x.x, bx[k].x);
         fx_mac(A2[q], x.x, bx[k].y);
         fx_mac(A2[q], x.y, bx[k].x);
@@ -498,19 +498,22 @@ __global__ void __launch_bounds__(128, TileShape<D, R, 8>::BLOCKS) recon_fixed_k
       if (nan) val = __longlong_as_double(0x7FF8000000000000ll);
       val = fma(val, scale, U0);
       if (active) Ufi[slot_of(f, q)] = val;
-      // positivity in FP32 with a margin of 1e-5 of rho E (its rounding: 1e-6); every lane shuffles
       const float x = fx_float(val);
-      const float rho = __shfl_sync(0xffffffffu, x, base), E = __shfl_sync(0xffffffffu, x, base + NV - 1);
-      float ke = 0.0f;
-#pragma unroll
-      for (int j = 0; j < D; ++j) {
-        const float mj = __shfl_sync(0xffffffffu, x, base + 1 + j);
-        ke += mj * mj;
-      }
-      const float rE = rho * E;
-      doubt = doubt || !(rho > 1e-30f && rE - 0.5f * ke > 1e-5f * rE && rE > 1e-30f);
+      low = fminf(low, x);
+      top = max(top, __float_as_uint(x) & 0x7FFFFFFFu);
     }
   }
+  // positivity of every point from those bounds, rho E - |m|^2 / 2 >= min rho min E - max |m|^2 / 2, with a margin
+  // of 1e-5 of rho E (its rounding: 1e-6)
+  const float rho = __shfl_sync(0xffffffffu, low, base), E = __shfl_sync(0xffffffffu, low, base + NV - 1);
+  float ke = 0.0f;
+#pragma unroll
+  for (int j = 0; j < D; ++j) {
+    const float m = __uint_as_float(__shfl_sync(0xffffffffu, top, base + 1 + j));
+    ke += m * m;
+  }
+  const float rE = rho * E;
+  const bool doubt = !(top < 0x7F800000u && rho > 1e-30f && E > 0.0f && rE > 1e-30f && rE - 0.5f * ke > 1e-5f * rE);
   if (a.guard_on && __any_sync(0xffffffffu, doubt && active)) {
     bool bad = false;
     for (int f = 0; f < NF; ++f)

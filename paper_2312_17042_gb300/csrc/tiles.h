@@ -29,15 +29,16 @@ struct TileShape {
   // memory latency of an SM (about 45 kB at the full rate) through the arithmetic. Measured, us a
   // launch (MC x NST): degree 4, 215 000 cells 10 x 3 123.7, 10 x 2 115.1, 6 x 3 117.7, 6 x 2 112.4; degree 6,
   // 180 000 cells 8 x 2 223.3, 8 x 3 230.2, 4 x 3 219.7, 4 x 4 237.4.
-  static constexpr int MC = E == 4 ? (R == 6 ? 4 : 6) : M <= 20 ? M : M % 4 == 0 ? 4 : 6;
-  static constexpr int NCH = M / MC, NMAX = E == 4 ? (R == 4 ? 2 : 3) : 3;
+  static constexpr int MC = E == 4 ? (R == 6 ? 4 : 6) : M == 12 ? 12 : M % 4 == 0 ? 4 : 6;
+  static constexpr int NCH = M / MC, NMAX = E == 4 ? (R == 4 ? 2 : 3) : 2;
   static constexpr int NST = NCH < NMAX ? NCH : NMAX;
   static constexpr int G = E == 4 ? MC : M % 4 == 0 ? 4 : 6;
   static constexpr int SLOTS = M < NF * ND ? M : NF * ND;
-  // FP64: face table [f][p][q][NKP], phi'_k as int2, rows of an even number of entries; 2D: the reversed edge
+  // FP64: face table (2D in shared memory; in 3D, where its 15 kB a block cost a third of the warps, read through
+  // L1) [f][p][q][NKP], phi'_k as int2, rows of an even number of entries; 2D: the reversed edge
   // swaps the stored points, one order (NP = 1)
   static constexpr int NP = D == 3 ? 6 : 1, NKP = (NK + 1) / 2 * 2;
-  static constexpr int PHI_BYTES = E == 8 ? NF * NP * NQ * NKP * 8 : 0;
+  static constexpr int PHI_BYTES = E == 8 && D == 2 ? NF * NP * NQ * NKP * 8 : 0;
   static constexpr int STAGE = CPW * MC * NK * E;
   // a warp's header: directional operators, then stencil ids
   static constexpr int HPD = CPW * NF * PDS * E, HDR = HPD + CPW * M * 4, DELTA = SLOTS * 32 * E;
