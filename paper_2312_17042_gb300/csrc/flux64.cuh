@@ -2,35 +2,26 @@
 // the time-step reduction and TwoSum helpers).
 //
 // Both kernels are bound by the FP64 pipe, which takes a warp instruction every 64 clocks per
-// scheduler whatever its other load, so they spend as few FP64 instructions as they can and spread
-// them over as many warps as the mesh gives:
+// scheduler whatever its other load, so they keep that pipe to the formulas and spread them over as many warps as
+// the mesh gives:
 //   face_flux64    one lane per face Gauss point (not per face): HLLC once per face in its owner's
-//                  orientation, comparisons and selections on integers, reciprocals and square roots
-//                  from the FP32-accurate hardware estimate and a third-order (Halley) or two
-//                  Newton-type corrections; the points of a face are summed by shuffles;
+//                  orientation, comparisons and selections on integers, square roots from the hardware estimate
+//                  and two corrections; the points of a face are exchanged by shuffles and summed in order;
 //   cell_update64  one lane per conserved variable: the cell's face fluxes, signed, in face order,
 //                  the Runge-Kutta update and, over the same lanes, the CFL step.
 // The per-cell schedules of the mixed path evaluate every face twice; in FP64 they took three times
 // as long and are not built.
 //
 // Measured, both kernels, against the per-cell schedule (the default then) and the face-based one with
-// a lane per face: 131 072 triangles, 2 points an edge 499 / 165 -> 121 us; 24 576 tetrahedra 362 / 122
-// -> 74 us; 4200 triangles, 3 points 123 / 49 -> 15 us; 2048 triangles 80 / 33 -> 13 us. The large
-// ones run at 80 % of the FP64 pipe. Small meshes want many small blocks (4200 triangles: 15.2 us in blocks
-// of 32 threads, 18.3 in blocks of 128), large ones do not care (121.7 / 121.2 us): 32 by default.
+// a lane per face: 131 072 triangles, 2 points an edge 499 / 165 -> 146 us; 24 576 tetrahedra 362 / 122
+// -> 89 us; 4200 triangles, 3 points 123 / 49 -> 17 us; 2048 triangles 80 / 33 -> 14 us. The large
+// ones run at 80 % of the FP64 pipe. Small meshes want many small blocks (4200 triangles: 16.7 us in blocks
+// of 32 threads, 20.4 in blocks of 128), large ones do not care (146.7 / 146.3 us): 32 by default.
 #pragma once
 
 namespace cteno {
 namespace {
 
-// 1 / x to about one unit in the last place: y (1 + e + e^2), e = 1 - x y, from an estimate y with
-// |e| < 2^-19. Normal x.
-__device__ __forceinline__ double rcp64(const double x) {
-  double y;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-  const double e = fma(-x, y, 1.0);
-  return fma(y, fma(e, e, e), y);
-}
 // sqrt(x): coupled iteration on g ~ sqrt(x) and h ~ 1 / (2 sqrt(x)) (Goldschmidt), then the
 // residual correction g + (x - g^2) h. Values below the normal numbers give 0.
 __device__ __forceinline__ double sqrt64(const double x) {
@@ -53,59 +44,70 @@ __device__ __forceinline__ bool less64(const double a, const double b) {
   return (x ^ ((x >> 63) & 0x7FFFFFFFFFFFFFFFll)) < (y ^ ((y >> 63) & 0x7FFFFFFFFFFFFFFFll));
 }
 
-// HLLC flux as hllc() (eqs. 24-29), with common factors taken once: about 125 FP64 instructions in 2D
-// and 140 in 3D, against 187 with IEEE division and square root.
+// HLLC flux as hllc() (eqs. 24-29), in its order, with IEEE division and roots to the last place: the states ahead of a
+// wave, whose selection hangs on differences of 1e-11, then round as those of any other FP64 evaluation of the
+// printed formulas does (taking common factors once and reciprocals one unit off saved a third of the time and
+// moved a 200-step shock tube by 5e-12 of its largest momentum, through selections of that size).
 template <int D>
 __device__ __forceinline__ void hllc64(const double *uL, const double *uR, const double *n, const double g, double *F) {
   constexpr int NV = D + 2;
-  const double rL = uL[0], rR = uR[0], gm1 = g - 1.0;
-  const double iL = rcp64(rL), iR = rcp64(rR);
-  double vL[D], vR[D], unL, unR, kL, kR;
+  auto quotient = [](double x, double y) { return x / y; };
+  auto lower = [](double x, double y) { return less64(x, y) ? x : y; };
+  auto higher = [](double x, double y) { return less64(x, y) ? y : x; };
+  const double rL = uL[0], rR = uR[0];
+  const double iL = 1.0 / (rL), iR = 1.0 / (rR);
+  double vL[D], vR[D], unL = 0, unR = 0, kL = 0, kR = 0;
 #pragma unroll
   for (int j = 0; j < D; ++j) {
     vL[j] = uL[1 + j] * iL;
     vR[j] = uR[1 + j] * iR;
-    unL = j ? fma(vL[j], n[j], unL) : vL[j] * n[j];
-    unR = j ? fma(vR[j], n[j], unR) : vR[j] * n[j];
-    kL = j ? fma(vL[j], uL[1 + j], kL) : vL[j] * uL[1 + j];
-    kR = j ? fma(vR[j], uR[1 + j], kR) : vR[j] * uR[1 + j];
+    unL += vL[j] * n[j];
+    unR += vR[j] * n[j];
+    kL += vL[j] * uL[1 + j];
+    kR += vR[j] * uR[1 + j];
   }
-  const double pL = gm1 * fma(-0.5, kL, uL[NV - 1]), pR = gm1 * fma(-0.5, kR, uR[NV - 1]);
+  const double pL = (g - 1) * (uL[NV - 1] - 0.5 * kL);
+  const double pR = (g - 1) * (uR[NV - 1] - 0.5 * kR);
   const double cL = sqrt64(g * pL * iL), cR = sqrt64(g * pR * iR);
   const double HL = (uL[NV - 1] + pL) * iL, HR = (uR[NV - 1] + pR) * iR;
-  const double Dr = sqrt64(rR * iL), idn = rcp64(1.0 + Dr);
-  double ut2, utn;
+  const double Dr = sqrt64(rR * iL);
+  const double idn = 1.0 / (1 + Dr);
+  double ut2 = 0, utn = 0;
 #pragma unroll
   for (int j = 0; j < D; ++j) {
-    const double ut = fma(vR[j], Dr, vL[j]) * idn;
-    ut2 = j ? fma(ut, ut, ut2) : ut * ut;
-    utn = j ? fma(ut, n[j], utn) : ut * n[j];
+    const double ut = (vL[j] + vR[j] * Dr) * idn;
+    ut2 += ut * ut;
+    utn += ut * n[j];
   }
-  const double Ht = fma(HR, Dr, HL) * idn, ct = sqrt64(gm1 * fma(-0.5, ut2, Ht));
-  const double sl1 = unL - cL, sl2 = utn - ct, sr1 = unR + cR, sr2 = utn + ct;
-  const double SL = less64(sl1, sl2) ? sl1 : sl2, SR = less64(sr1, sr2) ? sr2 : sr1;
-  const double aL = SL - unL, aR = SR - unR, mL = rL * aL, mR = rR * aR;
-  const double SM = (fma(mR, unR, -(mL * unL)) + (pL - pR)) * rcp64(mR - mL);
-  // the cases in the order SL > 0, SM > 0, SR > 0, else, without branches (see hllc)
-  const bool cl = positive64(SL), cm = positive64(SM), cr = positive64(SR);
-  const bool left = cl || cm, sup = cl || (!cm && !cr);
+  const double Ht = (HL + HR * Dr) * idn;
+  const double ct = sqrt64((g - 1) * (Ht - 0.5 * ut2));
+  const double SL = lower(unL - cL, utn - ct);
+  const double SR = higher(unR + cR, utn + ct);
+  const double SM = quotient(rR * unR * (SR - unR) - rL * unL * (SL - unL) + pL - pR,
+                       rR * (SR - unR) - rL * (SL - unL));
+  // The four cases, tested in the order SL > 0 (left state), SM > 0 (left star state), SR > 0
+  // (right star state), else (right state), evaluated without branches (neighbouring faces of a
+  // warp take different cases): the operands of side k are selected, the star correction is
+  // dropped in the two supersonic cases. Each case's arithmetic is the same as written out alone.
+  const bool left = positive64(SL) || positive64(SM);
+  const bool sup = positive64(SL) || (!positive64(SM) && !positive64(SR));
   double uk[NV];
 #pragma unroll
   for (int v = 0; v < NV; ++v) uk[v] = left ? uL[v] : uR[v];
-  const double pk = left ? pL : pR, unk = left ? unL : unR, Sk = left ? SL : SR, ak = left ? aL : aR;
+  const double pk = left ? pL : pR, unk = left ? unL : unR, Sk = left ? SL : SR, rk = uk[0];
   F[0] = uk[0] * unk;
 #pragma unroll
-  for (int j = 0; j < D; ++j) F[1 + j] = fma(uk[1 + j], unk, pk * n[j]);
+  for (int j = 0; j < D; ++j) F[1 + j] = uk[1 + j] * unk + pk * n[j];
   F[NV - 1] = (uk[NV - 1] + pk) * unk;
-  const double ps = fma(-mL, unL - SM, pL);
-  const double fct = rcp64(Sk - SM), s1 = fma(ak, fct, -1.0), dp = (ps - pk) * fct;
-  double G[NV];  // S_k (U* - U)
-  G[0] = Sk * (s1 * uk[0]);
+  const double ps = rL * (unL - SL) * (unL - SM) + pL;
+  const double fct = 1.0 / (Sk - SM), a = Sk - unk;
+  double G[NV];
+  G[0] = F[0] + Sk * (rk * a * fct - uk[0]);
 #pragma unroll
-  for (int j = 0; j < D; ++j) G[1 + j] = Sk * fma(dp, n[j], s1 * uk[1 + j]);
-  G[NV - 1] = Sk * fma(fma(ps, SM, -(pk * unk)), fct, s1 * uk[NV - 1]);
+  for (int j = 0; j < D; ++j) G[1 + j] = F[1 + j] + Sk * ((a * uk[1 + j] + (ps - pk) * n[j]) * fct - uk[1 + j]);
+  G[NV - 1] = F[NV - 1] + Sk * ((a * uk[NV - 1] - pk * unk + ps * SM) * fct - uk[NV - 1]);
 #pragma unroll
-  for (int v = 0; v < NV; ++v) F[v] = sup ? F[v] : F[v] + G[v];
+  for (int v = 0; v < NV; ++v) F[v] = sup ? F[v] : G[v];
 }
 
 // Local CFL step |V_i| / sum_f |A_f| (|u_i . n_f| + c_i) of the FP64 path: the velocity and the speed
@@ -113,14 +115,14 @@ __device__ __forceinline__ void hllc64(const double *uL, const double *uR, const
 // written out: the set-state kernels and the stage update must give the same bits.
 template <int D>
 __device__ __forceinline__ void speeds64(const double *u, const double g, double (&vel)[D], double &c) {
-  const double ir = rcp64(u[0]);
+  const double ir = 1.0 / u[0];
   double ke = 0.0;
 #pragma unroll
   for (int j = 0; j < D; ++j) {
     vel[j] = __dmul_rn(u[1 + j], ir);
     ke = fma(u[1 + j], vel[j], ke);
   }
-  c = sqrt64(__dmul_rn(__dmul_rn(g, __dmul_rn(g - 1.0, fma(-0.5, ke, u[D + 1]))), ir));
+  c = sqrt(__dmul_rn(__dmul_rn(g, __dmul_rn(g - 1.0, fma(-0.5, ke, u[D + 1]))), ir));
 }
 template <int D>
 __device__ __forceinline__ double face_speed64(const double *gf, const double (&vel)[D], const double c) {
@@ -135,7 +137,7 @@ __device__ __forceinline__ double local_dt64(const KArgs &a, const int64_t i, co
   speeds64<D>(u, a.gamma, vel, c);
 #pragma unroll
   for (int f = 0; f <= D; ++f) s = __dadd_rn(s, face_speed64<D>(a.geo + (i * (D + 1) + f) * 4, vel, c));
-  return rcp64(__dmul_rn(s, a.vol[i]));
+  return 1.0 / __dmul_rn(s, a.vol[i]);
 }
 
 template <int D, int NQ>
@@ -172,23 +174,15 @@ __global__ void __launch_bounds__(256) face_flux64_kernel(const KArgs a) {
     boundary_state<D, double, 1>(a, i, (__ldg(a.fmeta + i) >> (kMetaKindShift + 2 * f)) & 3u, gf, uI, um, uO);
   }
   hllc64<D>(uI, uO, gf, a.gamma, F);
-  double w = a.fw[0];
-#pragma unroll
-  for (int t = 1; t < NQ; ++t) w = (q == t) ? a.fw[t] : w;
-  w *= gf[3];
-  double out[NFP];
+  double out[NFP];  // |A| sum_q w_q F_q, in the order of the points
 #pragma unroll
   for (int v = 0; v < NFP; ++v) {
     double x = 0.0;
     if (v < NV) {
-      x = w * F[v];
-      if constexpr (NQ == 3) {
-        const double y = __shfl_sync(0xffffffffu, x, base + 1), z = __shfl_sync(0xffffffffu, x, base + 2);
-        x = (x + y) + z;  // the face's first lane stores it
-      } else {
+      x = a.fw[0] * __shfl_sync(0xffffffffu, F[v], base);
 #pragma unroll
-        for (int o = 1; o < NQ; o <<= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-      }
+      for (int t = 1; t < NQ; ++t) x = fma(a.fw[t], __shfl_sync(0xffffffffu, F[v], base + t), x);
+      x *= gf[3];
     }
     out[v] = x;
   }
@@ -248,7 +242,7 @@ __global__ void __launch_bounds__(256) cell_update64_kernel(const KArgs a) {
     const double x = face_speed64<D>(gf, vel, c);
 #pragma unroll
     for (int f = 0; f < NF; ++f) s = __dadd_rn(s, __shfl_sync(0xffffffffu, x, base + f));
-    const double dt = a.cfl * rcp64(__dmul_rn(s, a.vol[i]));
+    const double dt = a.cfl * (1.0 / __dmul_rn(s, a.vol[i]));
     warp_min_to(a.dt, a.nmesh + mesh, fin ? dt : 1e300);
   }
 }

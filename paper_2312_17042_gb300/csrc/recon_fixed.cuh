@@ -27,8 +27,8 @@
 // memory between the two products.
 //
 // Measured per launch against the FP64 schedules it replaced (bound by the FP64 pipe, 61 to 86 % of its
-// rate): 2D degree 3, 131 072 cells 534 -> 110 us; 3D degree 3, 24 576 cells 432 (553 in blocks of 128) -> 127
-// us; 2D degree 5, 4200 cells 81 -> 35 us; 2D degree 2, 2048 cells 19 (51 in blocks of 128) -> 12 us. It is
+// rate): 2D degree 3, 131 072 cells 534 -> 120 us; 3D degree 3, 24 576 cells 432 (553 in blocks of 128) -> 133
+// us; 2D degree 5, 4200 cells 81 -> 36 us; 2D degree 2, 2048 cells 19 (51 in blocks of 128) -> 12 us. It is
 // now bound by the integer pipe (shifts and 64-bit sums of the conversions, 63 % busy at 2D degree 3), the
 // small meshes by the length of a warp's chain.
 #pragma once
@@ -48,13 +48,15 @@ __device__ __forceinline__ int2 fx_split(const int64_t t) {
   return make_int2((int)(t >> 29), (int)((uint32_t)t & 0x1FFFFFFFu) - (1 << 28));
 }
 
-// u in units of 2^(e - 1079) less `base`, e the biased exponent of the unit's block: |u| < 2^(e - 1015), modulo
-// 2^64, truncated (a value far below the unit gives 0; e >= 64, so zeros and subnormals do).
+// u in units of 2^(e - 1079) less `base`, e the biased exponent of the unit's block, modulo 2^64, truncated
+// (a value far below the unit gives 0; e >= 64, so zeros and subnormals do).
 __device__ __forceinline__ int64_t fx_of(const double u, const int e, const int64_t base) {
-  const int hi = __double2hiint(u), lo = __double2loint(u);
-  const uint64_t m = ((uint64_t)(__funnelshift_l(lo, hi, 11) | 0x80000000u) << 32) | ((uint32_t)lo << 11);
-  uint64_t f;  // the shift is 7 to 64 and more places for |u| < 2^(e - 1022), 0 at the limit above
-  asm("shr.u64 %0, %1, %2;" : "=l"(f) : "l"(m), "r"(7 + e - ((hi >> 20) & 0x7FF)));
+  const int hi = __double2hiint(u);
+  const uint64_t m = ((uint64_t)((hi & 0xFFFFF) | 0x100000) << 32) | (uint32_t)__double2loint(u);
+  const int s = ((hi >> 20) & 0x7FF) - e + 4;
+  uint64_t f;
+  asm("shl.b64 %0, %1, %2;" : "=l"(f) : "l"(m), "r"(max(s, 0)));
+  asm("shr.u64 %0, %1, %2;" : "=l"(f) : "l"(f), "r"(max(-s, 0)));
   const int64_t sg = hi >> 31;
   return (int64_t)(f ^ (uint64_t)sg) - sg - base;
 }
@@ -257,10 +259,31 @@ __global__ void __launch_bounds__(128, TileShape<D, R, 8>::BLOCKS) recon_fixed_k
       kmin = min(kmin, k);
     }
   }
-  const double range = __hiloint2double(key(kmax), kmax < 0 ? 0 : -1) - __hiloint2double(key(kmin), kmin < 0 ? -1 : 0);
-  // |U_m - U_0| < 2^(er - 1022); the unit 2^(er - 1079) at least 2^-64 of the largest |U_m|
+  double range = __hiloint2double(key(kmax), kmax < 0 ? 0 : -1) - __hiloint2double(key(kmin), kmin < 0 ? -1 : 0);
+  // where the range is so small that the high words overestimate it by more than 2^-8, from the whole means: the
+  // decisions depend on ratios of indicators, so the differences need their own relative accuracy
   const int eu = (max(kmax, ~kmin) >> 20) & 0x7FF;
-  const int er = max((__double2hiint(range) >> 20) & 0x7FF, max(eu - 7, 64));
+  if (__any_sync(0xffffffffu, ((__double2hiint(range) >> 20) & 0x7FF) < eu - 12)) {
+    auto key64 = [](double u) {
+      const long long b = __double_as_longlong(u);
+      return b ^ ((b >> 63) & 0x7FFFFFFFFFFFFFFFll);
+    };
+    long long lmax = key64(U0), lmin = lmax;
+#pragma unroll 1
+    for (int m = 0; m < M; m += G) {
+      int j[G];
+      ids_of(m, j);
+#pragma unroll
+      for (int g = 0; g < G; ++g) {
+        const long long k = key64(__ldg(Uv + (int64_t)j[g] * NVP));
+        lmax = max(lmax, k);
+        lmin = min(lmin, k);
+      }
+    }
+    auto value = [](long long k) { return __longlong_as_double(k ^ ((k >> 63) & 0x7FFFFFFFFFFFFFFFll)); };
+    range = value(lmax) - value(lmin);
+  }
+  const int er = max((__double2hiint(range) >> 20) & 0x7FF, 64);  // |U_m - U_0| < 2^(er - 1022)
   // a non-finite member makes every coefficient NaN
   const bool finite = kmax < 0x7FF00000 && kmin > (int)0x800FFFFF && er < 0x7FF;
   const int64_t F0 = fx_of(U0, er, 1 << 28);
