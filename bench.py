@@ -259,15 +259,21 @@ def alu_peak(native):
     return {"fp64_tflops": round(f64, 3), "fp32_tflops": round(f32, 2)}
 
 
-def recon_kernel_name(dim, degree, scheme, precision, launch):
+def recon_kernel_name(dim, degree, scheme, precision, launch, characteristic=False):
     """Name of the reconstruction kernel a launch value selects."""
     args = f"{dim},{degree},{'float' if precision else 'double'},{SCHEMES[scheme]}"
-    if degree >= 4 and launch >= 1536:
-        return f"recon_high_kernel_occ<{degree},{SCHEMES[scheme]}> (64 registers) x{launch - 1536}"
+    if not precision and not characteristic:
+        return f"recon_fixed_kernel<{dim},{degree},{SCHEMES[scheme]}> x{min(launch % 1024, 128)}"
+    if degree >= 4 and not characteristic:
+        return f"recon_high_stream_kernel<{degree},{SCHEMES[scheme]}> x{min(launch % 512, 128)}"
     if degree >= 4:
         return f"recon_high_kernel<{degree},{'float' if precision else 'double'},{SCHEMES[scheme]}> x{launch - 1024}"
-    if 7168 < launch <= 7176 or 7200 < launch <= 7208:
-        return f"recon_pair_kernel<{args},{2 if launch < 7200 else 3} stages> x{32 * (launch % 32)}"
+    if launch > 11264:
+        return f"recon_tile_kernel<{dim},{degree},{SCHEMES[scheme]},1 variable> x{launch - 11264}"
+    if launch > 10240:
+        return f"recon_tile_kernel<{dim},{degree},{SCHEMES[scheme]},2 variables> x{launch - 10240}"
+    if launch > 7168:
+        return f"recon_tile_kernel<{dim},{degree},{SCHEMES[scheme]},2 variables> x{32 * min(launch % 32, 4)}"
     if 6144 < launch <= 6152:
         return f"recon_stream_cells_kernel<{args}> x{32 * (launch - 6144)}"
     if 5120 < launch <= 5136:
@@ -304,6 +310,8 @@ def ncu_traffic(key):
     degree = int(key.split(":")[1].split("_r")[1].split("_")[0])
     if degree >= 4 and not same("recon_high.cuh", "recon_high_cuh_sha256"):  # the degree 4-6 kernels
         return None
+    if int(key.rsplit(":", 1)[1]) > 7168 and not same("recon_tile.cuh", "recon_tile_cuh_sha256"):
+        return None
     return d.get("bytes_per_launch", {}).get(key)
 
 
@@ -335,18 +343,23 @@ def time_steps(native, s, steps, warmup, flush, torch, kernel_times=False):
 
 
 def roofline_of(case, scheme, degree, precision, launch, stats, recon_ms, peaks, peak_kind, alu):
-    """Roofline object of the reconstruction kernel (the dominant kernel of every workload): the
-    mixed path against the measured HBM copy bandwidth, the FP64 path against the measured FP64
-    FMA rate (it is bound by the FP64 pipe), both from algorithmic bytes / FLOPs per launch over
-    the mean launch time measured with CUDA events inside the replayed step graph."""
-    name = recon_kernel_name(case.dim, degree, scheme, precision, launch)
+    """Roofline object of the reconstruction kernel (the dominant kernel of every workload): against
+    the measured HBM copy bandwidth, from algorithmic bytes per launch over the mean launch time
+    measured with CUDA events inside the replayed step graph. The FP64 path's products run on the integer
+    pipe (its FLOPs, beside, are no fraction of the FP64 rate); only its characteristic reconstruction is
+    bound by the FP64 pipe, and reported against the measured FP64 FMA rate."""
+    characteristic = bool(case.extra.get("characteristic"))
+    name = recon_kernel_name(case.dim, degree, scheme, precision, launch, characteristic)
     gbs = stats[0] / (recon_ms * 1e-3) / 1e9
     key = f"{case.name}:{variant_name(scheme, degree, precision)}:{launch}"
-    if precision == 1 or alu is None:
-        return {"kernel": name, "bound": "hbm", "achieved": round(gbs, 1), "peak": peaks["hbm_gbs"],
-                "unit": "GB/s", "frac": round(gbs / peaks["hbm_gbs"], 4), "traffic": ncu_traffic(key),
-                "algorithmic_bytes_per_launch": stats[0], "launch_ms": round(recon_ms, 5),
-                "peak_source": f"MEASURED_PEAKS.json hbm_gbs ({peak_kind}, of measured)"}
+    if precision == 1 or not characteristic or alu is None:
+        out = {"kernel": name, "bound": "hbm", "achieved": round(gbs, 1), "peak": peaks["hbm_gbs"],
+               "unit": "GB/s", "frac": round(gbs / peaks["hbm_gbs"], 4), "traffic": ncu_traffic(key),
+               "algorithmic_bytes_per_launch": stats[0], "launch_ms": round(recon_ms, 5),
+               "peak_source": f"MEASURED_PEAKS.json hbm_gbs ({peak_kind}, of measured)"}
+        if precision == 0:
+            out["algorithmic_tflops"] = round(stats[2] / (recon_ms * 1e-3) / 1e12, 4)
+        return out
     tfl = stats[2] / (recon_ms * 1e-3) / 1e12
     return {"kernel": name, "bound": "alu", "achieved": round(tfl, 4), "peak": alu["fp64_tflops"],
             "unit": "TFLOP/s (FP64 FMA)", "frac": round(tfl / alu["fp64_tflops"], 4), "traffic": ncu_traffic(key),
@@ -394,7 +407,7 @@ def measure(native, case, scheme, degree, precision, stream, flush, torch, dist,
                    "achieved_gbs": round(stats[1] / (flux_ms * 1e-3) / 1e9, 1)}
     # per stage one reconstruction and one (or, face-based, two) flux/update launches; a
     # moving-shock boundary adds the time advance at the end of each step
-    out["gpu_launches"] = (3 * (1 + (2 if launch[1] >= 8192 else 1)) + (1 if "regions" in case.extra else 0)) * steps
+    out["gpu_launches"] = (3 * (1 + (2 if launch[1] >= 8192 or precision == 0 else 1)) + (1 if "regions" in case.extra else 0)) * steps
     if clk is not None:
         out["clocks"] = clk
     if e2e:
