@@ -75,9 +75,10 @@ typedef struct {
                            stencil with the weights of eq. 14, b = 4, on the CWENO split p_1) and
                            CTENO_SCHEME_TENO (Sec. 2.4: the cut-off of eqs. 19-23 without linear
                            coefficients, on the central least-squares polynomial itself) */
-  int precision;        /* CTENO_FP64: all arithmetic in FP64. CTENO_MIXED: reconstruction and
-                           flux in FP32; geometry, least-squares build, residual accumulation and
-                           the RK update in FP64 */
+  int precision;        /* CTENO_FP64: FP64 throughout (the inner products of the conserved-variable
+                           reconstruction as sums of 57-bit block fixed-point integers). CTENO_MIXED:
+                           reconstruction and flux in FP32; geometry, least-squares build, residual
+                           accumulation and the RK update in FP64 */
   int lam_gamma;        /* 1: scale-separation measure gamma_s carries the linear coefficient
                            lambda_s of eq. 18 (default, reproduces Tables 1-3); 0: as printed in
                            eq. 19 / Alg. 1-2 */

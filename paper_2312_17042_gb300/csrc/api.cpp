@@ -1086,9 +1086,6 @@ int cteno_autotune(cteno_ctx *ctx, int32_t *best_out) {
     for (int b : {kStagedCells + 32, kStagedCells + 64, kStagedCells + 128, kStagedLanes + 64,
                   kStagedLanes + 128, kStagedLanes + 256})
       if (recon_staged_smem(ctx->d, ctx->p.degree, 1, b) <= kMaxStagedSmem) rcand.push_back(b);
-  if (ctx->fp32 && ctx->p.degree <= 3)
-    for (int b : {32, 64, 128})
-      for (int k : {kTileLanes2, kTileLanes}) rcand.push_back(k + b);
   if (ctx->fp32 && ctx->hl) {
     const long long hs = recon_halo_smem(ctx->d, ctx->p.degree, ctx->hrec);
     if (hs <= kMaxStagedSmem) rcand.push_back(kHaloLanes);
@@ -1105,11 +1102,21 @@ int cteno_autotune(cteno_ctx *ctx, int32_t *best_out) {
   }
   if (ctx->p.characteristic)  // the variable-per-lane schedule only
     rcand = {kLaneSchedule + 64, kLaneSchedule + 128, kLaneSchedule + 256};
+  // a tile per warp, last: in 3D the lane schedules round the face values differently from the thread-per-cell
+  // ones (a polynomial at the point, a table), and these candidates speed up the former without
+  // deciding between the two
+  if (ctx->fp32 && ctx->p.degree <= 3 && !ctx->p.characteristic)
+    for (int b : {32, 64, 128})
+      for (int k : {kTileLanes2, kTileLanes}) rcand.push_back(k + b);
+  auto lane_values = [](int b) {
+    return (b >= kLaneSchedule && b < kStagedCells) || (b >= kStagedLanes && b < kStreamCells) || b > kTileLanes2;
+  };
   const int reps = 5;
   float best_r = 1e30f, best_f = 1e30f;
   int br = ctx->recon_block, bf = ctx->flux_block;
   const KArgs a = make_args(ctx, 1, 0);  // stage 1: reads U^n, writes U only
   for (int b : rcand) {  // the reconstruction writes only face states: no restore needed
+    if (ctx->d == 3 && b > kTileLanes2 && !lane_values(br)) continue;
     CK(launch_recon(ctx->d, ctx->p.degree, ctx->fp32, kscheme(ctx), a, b, ctx->stream));
     CK(cudaEventRecord(e0, ctx->stream));
     for (int r = 0; r < reps; ++r) CK(launch_recon(ctx->d, ctx->p.degree, ctx->fp32, kscheme(ctx), a, b, ctx->stream));

@@ -378,6 +378,13 @@ __device__ __forceinline__ void load16(const T *__restrict__ src, T *dst) {
 __device__ __forceinline__ void pdl_wait(const KArgs &a) {
   if (a.pdl) asm volatile("griddepcontrol.wait;" ::: "memory");
 }
+// A pointer to data that the previous kernel wrote, for read-only loads after pdl_wait: the compiler may move
+// such a load above the wait (they count as loads of constants) unless its address comes after it.
+template <typename P>
+__device__ __forceinline__ P *after_wait(P *p) {
+  asm volatile("" : "+l"(p) : : "memory");
+  return p;
+}
 // Launch a stage kernel, with the programmatic-serialisation attribute when a.pdl is set.
 inline void launch_stage_kernel(void (*kern)(KArgs), unsigned grid, unsigned block, size_t smem, cudaStream_t s,
                                 const KArgs &a) {

@@ -348,7 +348,7 @@ __global__ void __launch_bounds__(MINB ? 128 : 256, MINB ? MINB : 1) flux_kernel
   // reaches the time-step reduction
   const bool active = cell < N;
   const int64_t i = active ? cell : N - 1;
-  const T *__restrict__ Uf = (const T *)a.Uf;
+  const T *__restrict__ Uf = after_wait((const T *)a.Uf);
   const T *__restrict__ G = a.geo32;
   const T g = a.gamma32;
   const uint32_t meta = __ldg(a.fmeta + i);
@@ -440,7 +440,7 @@ __global__ void __launch_bounds__(256) face_flux_kernel(const KArgs a) {
   const int2 codes = __ldg(reinterpret_cast<const int2 *>(a.face) + e);  // owner, neighbour side
   const int64_t i = codes.x >> 2;
   const int f = codes.x & 3;
-  const T *__restrict__ Uf = (const T *)a.Uf;
+  const T *__restrict__ Uf = after_wait((const T *)a.Uf);
   const T *__restrict__ G = a.geo32;
   const T g = a.gamma32;
   T gf[4], uI[FB], uO[FB];
@@ -508,12 +508,13 @@ __global__ void __launch_bounds__(256) cell_update_kernel(const KArgs a) {
   const int4 cf4 = __ldg(reinterpret_cast<const int4 *>(a.cellface) + i);
   const int cfv[4] = {cf4.x, cf4.y, cf4.z, cf4.w};
   constexpr int NFP = (NV + 3) & ~3;
+  const T *__restrict__ Ff = after_wait((const T *)a.Ff);
 #pragma unroll
   for (int f = 0; f < NF; ++f) {
     const int64_t e = cfv[f] & 0x7FFFFFFF;
     const bool neg = cfv[f] < 0;
     T x[NFP];
-    load16<T, NFP>((const T *)a.Ff + e * NFP, x);
+    load16<T, NFP>(Ff + e * NFP, x);
 #pragma unroll
     for (int v = 0; v < NV; ++v) {
       const T c = neg ? -x[v] : x[v];

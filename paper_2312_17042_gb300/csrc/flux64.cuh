@@ -152,7 +152,7 @@ __global__ void __launch_bounds__(256) face_flux64_kernel(const KArgs a) {
   const int2 codes = __ldg(reinterpret_cast<const int2 *>(a.face) + e);  // owner, neighbour side
   const int64_t i = codes.x >> 2;
   const int f = codes.x & 3;
-  const double *__restrict__ Uf = (const double *)a.Uf;
+  const double *__restrict__ Uf = (const double *)after_wait((double *)a.Uf);
   auto state = [&](int64_t cell, int face_of, double *u) {
     const double *p = Uf + ((cell * NF + face_of) * NQ + q) * NV;
     if constexpr (D == 2) {
@@ -201,11 +201,12 @@ __global__ void __launch_bounds__(256) cell_update64_kernel(const KArgs a) {
   const int4 cf4 = __ldg(reinterpret_cast<const int4 *>(a.cellface) + i);
   const int cf[4] = {cf4.x, cf4.y, cf4.z, cf4.w};
   const int64_t at = i * NVP + v;
+  const double *__restrict__ Ff = after_wait((const double *)a.Ff);
   const double u = a.U[at];
   double acc = 0.0;  // sum_f |A_f| sum_q w_q F_q, signed for this cell
 #pragma unroll
   for (int f = 0; f < NF; ++f) {
-    const double x = __ldg((const double *)a.Ff + (int64_t)(cf[f] & 0x7FFFFFFF) * NFP + v);
+    const double x = __ldg(Ff + (int64_t)(cf[f] & 0x7FFFFFFF) * NFP + v);
     acc += cf[f] < 0 ? -x : x;
   }
   const int mesh = (a.nmesh > 1) ? mesh_of(a, i) : 0;

@@ -25,7 +25,7 @@ __global__ void __launch_bounds__(256) flux_lanes_kernel(const KArgs a) {
   const int64_t cell = ((int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * CPW + grp;
   const bool active = grp < CPW && cell < N;
   const int64_t i = active ? cell : N - 1;  // spare lanes shadow a valid cell, store nothing
-  const T *__restrict__ Uf = (const T *)a.Uf;
+  const T *__restrict__ Uf = after_wait((const T *)a.Uf);
   const T *__restrict__ G = a.geo32;
   const T g = a.gamma32;
   const uint32_t meta = __ldg(a.fmeta + i);

@@ -228,7 +228,7 @@ __global__ void __launch_bounds__(128, TileShape<D, R, 8>::BLOCKS) recon_fixed_k
     if (S::PHI_BYTES) arrived(tbar, 0, 0, 0);
     return;
   }
-  const double *__restrict__ Uv = a.U + v;
+  const double *__restrict__ Uv = after_wait(a.U) + v;
   const int32_t *__restrict__ sti = reinterpret_cast<const int32_t *>(wmem + S::HPD) + slot * M;
   const double U0 = __ldg(Uv + i * NVP);
   auto ids_of = [&](int m, int (&j)[G]) {

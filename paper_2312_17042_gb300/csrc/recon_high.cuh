@@ -282,7 +282,7 @@ __global__ void __launch_bounds__(128, TileShape<2, R, 4>::BLOCKS) recon_high_st
     __syncwarp();
     return false;
   };
-  const float2 *__restrict__ Uv = reinterpret_cast<const float2 *>(a.U32) + v;
+  const float2 *__restrict__ Uv = reinterpret_cast<const float2 *>(after_wait(a.U32)) + v;
   const int32_t *__restrict__ sti = reinterpret_cast<const int32_t *>(wmem + S::HPD) + slot * M;
   const float2 own = __ldg(Uv + i * NVP);
   const float U0 = own.x, L0 = own.y;

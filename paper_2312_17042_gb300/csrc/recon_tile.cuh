@@ -116,7 +116,7 @@ __global__ void __launch_bounds__(128, TileDims<D, R, VPL>::BLOCKS) recon_tile_k
   if (a.test_wait_ns && !arrived(&bar[1 + NST], 0, 0, NST, a.test_wait_ns)) return;
   using Pairs = typename std::conditional<VPL == 2, float4, float2>::type;      // (hi, lo) of a lane's variables
   constexpr int NU = L::NVP / VPL;
-  const Pairs *__restrict__ Uq = reinterpret_cast<const Pairs *>(a.U32) + s;
+  const Pairs *__restrict__ Uq = reinterpret_cast<const Pairs *>(after_wait(a.U32)) + s;
   const int32_t *__restrict__ sti = reinterpret_cast<const int32_t *>(wmem + Q::HPD) + slot * M;
   float *const sdel = reinterpret_cast<float *>(dmem) + VPL * lane;
   const Pairs own = __ldg(Uq + i * NU);
