@@ -625,6 +625,10 @@ int cteno_lsq_build(cteno_ctx *ctx) {
   CK(cudaMemsetAsync(ctx->derr, 0, sizeof(int), ctx->stream));
   CK(cudaMemsetAsync(ctx->guard, 0, sizeof(unsigned long long), ctx->stream));
   CK(cudaMemsetAsync(ctx->U, 0, sizeof(double) * nvp * N, ctx->stream));
+  // U^n, the RK4 sum and the steps too: cteno_autotune times a stage before any step has written them
+  CK(cudaMemsetAsync(ctx->Un, 0, sizeof(double) * nvp * N, ctx->stream));
+  if (ctx->Acc) CK(cudaMemsetAsync(ctx->Acc, 0, sizeof(double) * nvp * N, ctx->stream));
+  CK(cudaMemsetAsync(ctx->dt, 0, sizeof(double) * 2 * nmesh, ctx->stream));
   if (ctx->U32) CK(cudaMemsetAsync(ctx->U32, 0, 2 * sizeof(float) * nvp * N, ctx->stream));
   SetupArgs s{};
   s.N = N;
