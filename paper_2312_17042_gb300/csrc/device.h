@@ -379,7 +379,8 @@ __device__ __forceinline__ void pdl_wait(const KArgs &a) {
   if (a.pdl) asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 // A pointer to data that the previous kernel wrote, for read-only loads after pdl_wait: the compiler may move
-// such a load above the wait (they count as loads of constants) unless its address comes after it.
+// such a load above the wait (they count as loads of constants) unless its address comes after it. Every kernel
+// launched by launch_stage_kernel takes the state, the face states and the face fluxes through it.
 template <typename P>
 __device__ __forceinline__ P *after_wait(P *p) {
   asm volatile("" : "+l"(p) : : "memory");

@@ -319,15 +319,24 @@ __device__ __forceinline__ void cweno_weights(float SI0, const float *SId, uint3
   for (int f = 0; f < NF; ++f) wd[f] *= inv;
 }
 
+// The state that the previous kernel wrote, FP64 means or (T = float) their FP32 pairs: every read-only load of
+// it starts from this pointer, taken behind pdl_wait (see after_wait).
+template <typename T>
+__device__ __forceinline__ const T *state_after_wait(const KArgs &a) {
+  if constexpr (sizeof(T) == 4) return after_wait((const T *)a.U32);
+  else return after_wait((const T *)a.U);
+}
+
 // Own cell means of cell i: FP64, or (mixed path) the FP32 pair hi + lo of every FP64 value, so
 // that U_m - U_0 = (hi_m - hi_0) + (lo_m - lo_0) keeps FP64 accuracy in FP32 arithmetic.
+// Us: state_after_wait, here and below.
 template <int D, typename T>
-__device__ __forceinline__ void cell_own(const KArgs &a, const int64_t i, T (&U0)[Lay<D>::NV],
+__device__ __forceinline__ void cell_own(const T *Us, const int64_t i, T (&U0)[Lay<D>::NV],
                                          float (&L0)[Lay<D>::NV]) {
   constexpr int NV = Lay<D>::NV, NVP = Lay<D>::NVP;
   if constexpr (sizeof(T) == 4) {
     float hl[2 * NVP];
-    load16<float, 2 * NVP>(a.U32 + i * 2 * NVP, hl);
+    load16<float, 2 * NVP>(Us + i * 2 * NVP, hl);
 #pragma unroll
     for (int v = 0; v < NV; ++v) {
       U0[v] = hl[2 * v];
@@ -335,7 +344,7 @@ __device__ __forceinline__ void cell_own(const KArgs &a, const int64_t i, T (&U0
     }
   } else {
     double u[NVP];
-    load16<double, NVP>(a.U + i * NVP, u);
+    load16<double, NVP>(Us + i * NVP, u);
 #pragma unroll
     for (int v = 0; v < NV; ++v) {
       U0[v] = (T)u[v];
@@ -346,17 +355,17 @@ __device__ __forceinline__ void cell_own(const KArgs &a, const int64_t i, T (&U0
 
 // U_j - U_0 for every variable (eq. 10), from member j's record.
 template <int D, typename T>
-__device__ __forceinline__ void cell_delta(const KArgs &a, const int64_t j, const T (&U0)[Lay<D>::NV],
+__device__ __forceinline__ void cell_delta(const T *Us, const int64_t j, const T (&U0)[Lay<D>::NV],
                                            const float (&L0)[Lay<D>::NV], T *du) {
   constexpr int NV = Lay<D>::NV, NVP = Lay<D>::NVP;
   if constexpr (sizeof(T) == 4) {
     float hl[2 * NVP];
-    load16<float, 2 * NVP>(a.U32 + j * 2 * NVP, hl);
+    load16<float, 2 * NVP>(Us + j * 2 * NVP, hl);
 #pragma unroll
     for (int v = 0; v < NV; ++v) du[v] = (T)((hl[2 * v] - (float)U0[v]) + (hl[2 * v + 1] - L0[v]));
   } else {
     double u[NVP];
-    load16<double, NVP>(a.U + j * NVP, u);
+    load16<double, NVP>(Us + j * NVP, u);
 #pragma unroll
     for (int v = 0; v < NV; ++v) du[v] = (T)(u[v] - (double)U0[v]);
   }
@@ -368,7 +377,7 @@ __device__ __forceinline__ void cell_delta(const KArgs &a, const int64_t j, cons
 // points with the positivity guard. Pdi, sti: the cell's directional operators and stencil ids in
 // global memory (SH = false) or in a shared-memory copy (SH = true).
 template <int D, int R, typename T, int SCHEME, bool SH>
-__device__ __forceinline__ void cell_finish(const KArgs &a, const int64_t i,
+__device__ __forceinline__ void cell_finish(const KArgs &a, const T *Us, const int64_t i,
                                             T (&ao)[Shape<D, R>::NK][Lay<D>::NV], const T (&U0)[Lay<D>::NV],
                                             const float (&L0)[Lay<D>::NV], const T *__restrict__ Pdi,
                                             const int32_t *__restrict__ sti, const T *__restrict__ sPhi) {
@@ -378,7 +387,7 @@ __device__ __forceinline__ void cell_finish(const KArgs &a, const int64_t i,
   constexpr int NK = S::NK, NP = S::NP;
   constexpr bool F32 = sizeof(T) == 4;
   const int64_t N = a.N;
-  auto delta = [&](int64_t j, T *du) { cell_delta<D, T>(a, j, U0, L0, du); };
+  auto delta = [&](int64_t j, T *du) { cell_delta<D, T>(Us, j, U0, L0, du); };
 
   // directional coefficients (degree 1): members of face f are the next slots of the list
   const uint32_t info = __ldg(a.cinfo + i);
@@ -569,7 +578,7 @@ __device__ __forceinline__ void cell_finish(const KArgs &a, const int64_t i,
 }
 
 template <int D, int R, typename T, int SCHEME, bool SH>
-__device__ __forceinline__ void recon_cell(const KArgs &a, const int64_t i, const T *__restrict__ Pci,
+__device__ __forceinline__ void recon_cell(const KArgs &a, const T *Us, const int64_t i, const T *__restrict__ Pci,
                                            const T *__restrict__ Pdi, const int32_t *__restrict__ sti,
                                            const T *__restrict__ sPhi) {
   using S = Shape<D, R>;
@@ -579,7 +588,7 @@ __device__ __forceinline__ void recon_cell(const KArgs &a, const int64_t i, cons
   constexpr int CH = Vec16<T>::n;
   T U0[NV];
   float L0[NV];
-  cell_own<D, T>(a, i, U0, L0);
+  cell_own<D, T>(Us, i, U0, L0);
 
   // 1-2: central coefficients a_opt = P_c (U_m - U_0), streaming the member-major record
   T ao[NK][NV];
@@ -602,13 +611,13 @@ __device__ __forceinline__ void recon_cell(const KArgs &a, const int64_t i, cons
           const int4 t4 = load_i4<SH>(sti + m);
           ids[0] = t4.x; ids[1] = t4.y; ids[2] = t4.z; ids[3] = t4.w;
         }
-        cell_delta<D, T>(a, ids[m % 4], U0, L0, du);
+        cell_delta<D, T>(Us, ids[m % 4], U0, L0, du);
       }
 #pragma unroll
       for (int v = 0; v < NV; ++v) ao[k][v] += pb[e % CH] * du[v];
     }
   }
-  cell_finish<D, R, T, SCHEME, SH>(a, i, ao, U0, L0, Pdi, sti, sPhi);
+  cell_finish<D, R, T, SCHEME, SH>(a, Us, i, ao, U0, L0, Pdi, sti, sPhi);
 }
 
 // MINB > 0: register-capped variant (at most 128 threads per block, MINB blocks per SM), which the
@@ -636,7 +645,7 @@ __global__ void __launch_bounds__(MINB ? 128 : 256, MINB ? MINB : 1) recon_kerne
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= N) return;
 
-  recon_cell<D, R, T, SCHEME, false>(a, i, (const T *)a.Pc + i * (int64_t)(M * NK),
+  recon_cell<D, R, T, SCHEME, false>(a, state_after_wait<T>(a), i, (const T *)a.Pc + i * (int64_t)(M * NK),
                                      (const T *)a.Pd + i * (int64_t)(NF * PDS), a.st + i * M, sPhi);
 
   // CFL time step bookkeeping at the first stage of a step: dt[next] -> dt[cur]
@@ -1116,9 +1125,9 @@ __device__ __forceinline__ void lane_finish(const KArgs &a, const int64_t i, con
 // every lane of the warp calls it (inactive lanes with a clamped valid cell i) because the
 // positivity guard exchanges values with shuffles. Operator pointers as for recon_cell. HALO:
 // sti holds the cell's uint16 local indices (members, then the cell itself) into `halo`, the
-// shared-memory FP32 (hi, lo) records of its tile's distinct stencil members.
+// shared-memory FP32 (hi, lo) records of its tile's distinct stencil members, and Us is not read.
 template <int D, int R, typename T, int SCHEME, bool SH, bool HALO = false, bool CHR = false>
-__device__ __forceinline__ void recon_lane(const KArgs &a, const int64_t i, const bool active, const int v,
+__device__ __forceinline__ void recon_lane(const KArgs &a, const T *Us, const int64_t i, const bool active, const int v,
                                            const int base, const T *__restrict__ Pci,
                                            const T *__restrict__ Pdi, const void *__restrict__ sti_,
                                            const T *__restrict__ sPhi, const float *__restrict__ halo = nullptr) {
@@ -1139,11 +1148,11 @@ __device__ __forceinline__ void recon_lane(const KArgs &a, const int64_t i, cons
     U0 = h.x;
     L0 = h.y;
   } else if constexpr (F32) {
-    const float2 h = __ldg(reinterpret_cast<const float2 *>(a.U32) + i * NVP + v);
+    const float2 h = __ldg(reinterpret_cast<const float2 *>(Us) + i * NVP + v);
     U0 = h.x;
     L0 = h.y;
   } else {
-    U0 = (T)__ldg(a.U + i * NVP + v);
+    U0 = (T)__ldg(Us + i * NVP + v);
     L0 = 0.0f;
   }
   auto delta = [&](int64_t j) -> T {
@@ -1151,10 +1160,10 @@ __device__ __forceinline__ void recon_lane(const KArgs &a, const int64_t i, cons
       const float2 h = reinterpret_cast<const float2 *>(halo)[(int)j * NVP + v];
       return (h.x - (float)U0) + (h.y - L0);
     } else if constexpr (F32) {
-      const float2 h = __ldg(reinterpret_cast<const float2 *>(a.U32) + j * NVP + v);
+      const float2 h = __ldg(reinterpret_cast<const float2 *>(Us) + j * NVP + v);
       return (h.x - (float)U0) + (h.y - L0);
     } else {
-      return (T)(__ldg(a.U + j * NVP + v) - (double)U0);
+      return (T)(__ldg(Us + j * NVP + v) - (double)U0);
     }
   };
   constexpr int IDV = HALO ? 8 : 4;  // ids per 16-byte load
@@ -1253,8 +1262,8 @@ __global__ void __launch_bounds__(256) recon_lanes_kernel(const KArgs a) {
   const bool active = grp < CPW && cell < N;
   const int64_t i = active ? cell : N - 1;  // spare lanes shadow a valid cell
 
-  recon_lane<D, R, T, SCHEME, false, false, CHR>(a, i, active, v, base, (const T *)a.Pc + i * (int64_t)(M * NK),
-                                     (const T *)a.Pd + i * (int64_t)(NF * PDS), a.st + i * M, sPhi);
+  recon_lane<D, R, T, SCHEME, false, false, CHR>(a, state_after_wait<T>(a), i, active, v, base,
+                                     (const T *)a.Pc + i * (int64_t)(M * NK), (const T *)a.Pd + i * (int64_t)(NF * PDS), a.st + i * M, sPhi);
   if (a.dt_swap && blockIdx.x == 0)
     for (int t = threadIdx.x; t < a.nmesh; t += blockDim.x) {
       a.dt[t] = a.dt[a.nmesh + t];
@@ -1347,6 +1356,7 @@ __global__ void __launch_bounds__(256) recon_staged_kernel(const KArgs a) {
   // the operator records do not depend on the previous kernel: their copies were issued above;
   // the states it writes (and the face states it may still read) are touched only after this
   pdl_wait(a);
+  const T *const Us = state_after_wait<T>(a);
   // CFL time step bookkeeping at the first stage of a step: dt[next] -> dt[cur]
   if (a.dt_swap && blockIdx.x == 0)
     for (int t = threadIdx.x; t < a.nmesh; t += blockDim.x) {
@@ -1374,13 +1384,13 @@ __global__ void __launch_bounds__(256) recon_staged_kernel(const KArgs a) {
       const int slot = (int)(threadIdx.x >> 5) * CPW + grp;
       const bool active = grp < CPW && slot < nvalid;
       const int ls = active ? slot : nvalid - 1;  // spare lanes shadow a valid cell of the tile
-      recon_lane<D, R, T, SCHEME, true>(a, c0 + ls, active, lane - grp * NV, grp * NV,
+      recon_lane<D, R, T, SCHEME, true>(a, Us, c0 + ls, active, lane - grp * NV, grp * NV,
                                         sPc(s) + ls * (M * NK), sPd(s) + ls * (NF * PDS),
                                         sSt(s) + ls * M, sPhi);
     } else {
       const int slot = threadIdx.x;
       if (slot < nvalid)
-        recon_cell<D, R, T, SCHEME, true>(a, c0 + slot, sPc(s) + slot * (M * NK),
+        recon_cell<D, R, T, SCHEME, true>(a, Us, c0 + slot, sPc(s) + slot * (M * NK),
                                           sPd(s) + slot * (NF * PDS), sSt(s) + slot * M, sPhi);
     }
     __syncthreads();  // every thread is done with stage s
@@ -1463,7 +1473,7 @@ __global__ void __launch_bounds__(kHaloWarps * 32) recon_halo_kernel(const KArgs
     const bool active = grp < CPW && slot < nvalid;
     const int ls = active ? slot : nvalid - 1;  // spare lanes shadow a valid cell of the tile
     unsigned char *b = base(s);
-    recon_lane<D, R, T, SCHEME, true, true>(a, c0 + ls, active, lane - grp * NV, grp * NV,
+    recon_lane<D, R, T, SCHEME, true, true>(a, nullptr, c0 + ls, active, lane - grp * NV, grp * NV,
                                             reinterpret_cast<const T *>(b) + ls * (M * NK),
                                             reinterpret_cast<const T *>(b + o_pd) + ls * (NF * PDS),
                                             b + o_li + (size_t)ls * LI, sPhi,
@@ -1670,6 +1680,7 @@ __global__ void __launch_bounds__(512, 1) recon_stream_kernel(const KArgs a) {
     }
   }
   pdl_wait(a);  // states written by the previous stage's update
+  const float2 *const Us = reinterpret_cast<const float2 *>(state_after_wait<T>(a));
   if (a.dt_swap && blockIdx.x == 0)
     for (int t = threadIdx.x; t < a.nmesh; t += blockDim.x) {
       a.dt[t] = a.dt[a.nmesh + t];
@@ -1684,7 +1695,7 @@ __global__ void __launch_bounds__(512, 1) recon_stream_kernel(const KArgs a) {
     const bool active = grp < CPW && grp < nvalid;
     const int g = active ? grp : nvalid - 1;  // spare lanes shadow a valid cell of the tile
     const int64_t i = c0 + g;
-    const float2 own = __ldg(reinterpret_cast<const float2 *>(a.U32) + i * NVP + v);
+    const float2 own = __ldg(Us + i * NVP + v);
     const T U0 = own.x;
     const float L0 = own.y;
     const uint32_t info = __ldg(a.cinfo + i);
@@ -1695,7 +1706,7 @@ __global__ void __launch_bounds__(512, 1) recon_stream_kernel(const KArgs a) {
     const T *__restrict__ Pd_s = reinterpret_cast<const T *>(hdr(it)) + g * (NF * PDS);
     const int32_t *__restrict__ st_s = reinterpret_cast<const int32_t *>(hdr(it) + Q::HPD) + g * M;
     auto delta = [&](int32_t j) -> T {
-      const float2 h = __ldg(reinterpret_cast<const float2 *>(a.U32) + (int64_t)j * NVP + v);
+      const float2 h = __ldg(Us + (int64_t)j * NVP + v);
       return (h.x - U0) + (h.y - L0);
     };
 
@@ -1709,7 +1720,7 @@ __global__ void __launch_bounds__(512, 1) recon_stream_kernel(const KArgs a) {
 #pragma unroll
       for (int mm = 0; mm < MC; mm += 4) {
         const int4 j4 = *reinterpret_cast<const int4 *>(st_s + c * MC + mm);
-        const float2 *u = reinterpret_cast<const float2 *>(a.U32) + v;
+        const float2 *u = Us + v;
         nx[mm] = __ldg(u + (int64_t)j4.x * NVP);
         nx[mm + 1] = __ldg(u + (int64_t)j4.y * NVP);
         nx[mm + 2] = __ldg(u + (int64_t)j4.z * NVP);
@@ -1876,6 +1887,7 @@ __global__ void __launch_bounds__(256, 1) recon_stream_cells_kernel(const KArgs 
     }
   }
   pdl_wait(a);  // states written by the previous stage's update
+  const T *const Us = state_after_wait<T>(a);
   if (a.dt_swap && blockIdx.x == 0)
     for (int t = threadIdx.x; t < a.nmesh; t += blockDim.x) {
       a.dt[t] = a.dt[a.nmesh + t];
@@ -1889,7 +1901,7 @@ __global__ void __launch_bounds__(256, 1) recon_stream_cells_kernel(const KArgs 
     const int64_t i = active ? i0 : N - 1;  // lanes past the last cell shadow it and store nothing
     T U0[NV];
     float L0[NV];
-    cell_own<D, T>(a, i, U0, L0);
+    cell_own<D, T>(Us, i, U0, L0);
     const int32_t *__restrict__ sti = a.st + i * M;
     T ao[NK][NV];
 #pragma unroll
@@ -1900,10 +1912,10 @@ __global__ void __launch_bounds__(256, 1) recon_stream_cells_kernel(const KArgs 
     for (int c = 0; c < NCH; ++c, ++q) {
       const int4 j4 = load_i4<false>(sti + c * MC);
       T du[MC][NV];
-      cell_delta<D, T>(a, j4.x, U0, L0, du[0]);
-      cell_delta<D, T>(a, j4.y, U0, L0, du[1]);
-      cell_delta<D, T>(a, j4.z, U0, L0, du[2]);
-      cell_delta<D, T>(a, j4.w, U0, L0, du[3]);
+      cell_delta<D, T>(Us, j4.x, U0, L0, du[0]);
+      cell_delta<D, T>(Us, j4.y, U0, L0, du[1]);
+      cell_delta<D, T>(Us, j4.z, U0, L0, du[2]);
+      cell_delta<D, T>(Us, j4.w, U0, L0, du[3]);
       if (!wait_all(&pbar[q % NST], (uint32_t)((q / NST) & 1))) {
         give_up(q, qi);
         return;
@@ -1921,7 +1933,7 @@ __global__ void __launch_bounds__(256, 1) recon_stream_cells_kernel(const KArgs 
       ++qi;
     }
     if (active)
-      cell_finish<D, R, T, SCHEME, false>(a, i, ao, U0, L0, (const T *)a.Pd + i * (int64_t)(NF * PDS), sti, sPhi);
+      cell_finish<D, R, T, SCHEME, false>(a, Us, i, ao, U0, L0, (const T *)a.Pd + i * (int64_t)(NF * PDS), sti, sPhi);
   }
 }
 

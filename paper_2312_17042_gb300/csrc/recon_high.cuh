@@ -116,6 +116,7 @@ __device__ __forceinline__ void recon_high_body(const KArgs &a) {
   constexpr bool F32 = sizeof(T) == 4;
   static_assert((G * NK) % CH == 0 && NDP % CH == 0 && PDS % CH == 0, "16-byte aligned records");
   pdl_wait(a);  // the state written by the previous stage's update
+  const T *const Us = state_after_wait<T>(a);
   const int lane = threadIdx.x & 31;
   const int grp = lane / NV, v = lane - grp * NV, base = grp * NV;
   const int64_t N = a.N;
@@ -127,19 +128,19 @@ __device__ __forceinline__ void recon_high_body(const KArgs &a) {
   T U0;
   float L0;
   if constexpr (F32) {
-    const float2 h = __ldg(reinterpret_cast<const float2 *>(a.U32) + i * NVP + v);
+    const float2 h = __ldg(reinterpret_cast<const float2 *>(Us) + i * NVP + v);
     U0 = h.x;
     L0 = h.y;
   } else {
-    U0 = __ldg(a.U + i * NVP + v);
+    U0 = __ldg(Us + i * NVP + v);
     L0 = 0.0f;
   }
   auto delta = [&](int64_t j) -> T {  // U_j - U_0 of variable v (eq. 10)
     if constexpr (F32) {
-      const float2 h = __ldg(reinterpret_cast<const float2 *>(a.U32) + j * NVP + v);
+      const float2 h = __ldg(reinterpret_cast<const float2 *>(Us) + j * NVP + v);
       return (h.x - (float)U0) + (h.y - L0);
     } else {
-      return __ldg(a.U + j * NVP + v) - U0;
+      return __ldg(Us + j * NVP + v) - U0;
     }
   };
   const int32_t *__restrict__ sti = a.st + i * M;
