@@ -458,8 +458,8 @@ __global__ void __launch_bounds__(128, TileShape<D, R, 8>::BLOCKS) recon_fixed_k
       bits = select_fp64<NF>(SI0, SId, adm, stn, SCHEME, a.ctenoz_form, a.lam_gamma, a.lam1, lams, a.eps, a.C_T);
     }
   }
-  if (!(bits & 1u)) {  // the mean of the selected directional polynomials
-    scale = 1.0 / (double)__popc(bits >> 1);
+  if (!(bits & 1u)) {  // the mean of the selected directional polynomials (none selected: p = 0)
+    scale = bits ? 1.0 / (double)__popc(bits >> 1) : 1.0;
 #pragma unroll
     for (int k = 0; k < NK; ++k) ao[k] = 0.0;
 #pragma unroll

@@ -1,0 +1,45 @@
+"""The FP64 path at the limits of what it accepts, against the FP64 oracle: its reconstruction takes the central
+inner products in integers and its flux compares wave speeds by their bits, and neither may show."""
+from __future__ import annotations
+
+import numpy as np
+import pytest
+
+import workloads as W
+from tests.test_gpu_parity import _native, _ragged, _relerr, _solver
+
+pytestmark = pytest.mark.gpu
+
+MESHES = {
+    "tri-r2": (lambda: W.shock_tube_2d(23, 7), 2),
+    "tri-r3": (lambda: W.density_wave_2d(12), 3),
+    "tri-r4": (lambda: W.density_wave_2d(18), 4),
+    "tri-r5": (lambda: W.shock_tube_2d(21, 17), 5),
+    "tri-r6": (lambda: W.density_wave_2d(21), 6),
+    "tet-r2": (lambda: W.density_wave_3d(6), 2),
+    "tet-r3": (lambda: _ragged(W.blast_3d(6), 5), 3),
+}
+
+
+@pytest.mark.parametrize("guard", [0, 1])
+@pytest.mark.parametrize("name", list(MESHES))
+def test_cut_off_that_drops_every_stencil(name, guard):
+    """TENO with C_T = 0.5: in smooth flow every chi_s is about 1 / s_t, no stencil is kept, and the face states
+    are the mean (p = 0 added to U_0), with no help of the positivity guard."""
+    native = _native()
+    from oracle import Oracle
+    make, degree = MESHES[name]
+    wl = make()
+    d = wl.mesh.dim
+    o = Oracle(wl.mesh, degree=degree, scheme=3, C_T=0.5, guard=guard)
+    o.set_state(wl.U0)
+    o.residual()
+    s = _solver(native, [wl.mesh], d, degree=degree, scheme=3, C_T=0.5, positivity_guard=guard)
+    native.cteno_record_flags(s.ctx, True)
+    s.set_state(wl.U0)
+    s.stage(0, 0.0)
+    got, flags, count = native.cteno_get_face_states(s.ctx, 0), native.cteno_get_flags(s.ctx, 0), s.sync()
+    s.close()
+    assert (o.flags() == 0).any()
+    assert np.array_equal(flags, o.flags()) and count == o.nguard()
+    assert _relerr(got.reshape(-1, d + 2).T, o.face_states().reshape(-1, d + 2).T) < 1e-12
