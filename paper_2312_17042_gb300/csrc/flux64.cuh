@@ -34,14 +34,24 @@ __device__ __forceinline__ double sqrt64(const double x) {
   g = fma(fma(-g, g, x), h, g);
   return (__double2hiint(x) & 0x7FFFFFFF) < 0x00100000 ? 0.0 : g;
 }
-// x > 0, a < b, on integers.
+// x > 0, and fmin(a, b), fmax(a, b) with their rule for NaN (the other operand: a side with a negative pressure has
+// no speed of sound, and the wave speeds are then those of the other side and of the Roe average), on integers.
 __device__ __forceinline__ bool positive64(const double x) {
   const int h = __double2hiint(x);
   return (h > 0 && h <= 0x7FF00000) || (h == 0 && __double2loint(x) != 0);
 }
+__device__ __forceinline__ bool nan64(const double x) {  // of a result: its quiet bit is in the high word
+  return (__double2hiint(x) & 0x7FFFFFFF) > 0x7FF00000;
+}
 __device__ __forceinline__ bool less64(const double a, const double b) {
   const long long x = __double_as_longlong(a), y = __double_as_longlong(b);
   return (x ^ ((x >> 63) & 0x7FFFFFFFFFFFFFFFll)) < (y ^ ((y >> 63) & 0x7FFFFFFFFFFFFFFFll));
+}
+__device__ __forceinline__ double lower64(const double a, const double b) {
+  return (less64(a, b) || nan64(b)) && !nan64(a) ? a : b;
+}
+__device__ __forceinline__ double higher64(const double a, const double b) {
+  return (less64(b, a) || nan64(b)) && !nan64(a) ? a : b;
 }
 
 // HLLC flux as hllc() (eqs. 24-29), in its order, with IEEE division and roots to the last place: the states ahead of a
@@ -52,8 +62,6 @@ template <int D>
 __device__ __forceinline__ void hllc64(const double *uL, const double *uR, const double *n, const double g, double *F) {
   constexpr int NV = D + 2;
   auto quotient = [](double x, double y) { return x / y; };
-  auto lower = [](double x, double y) { return less64(x, y) ? x : y; };
-  auto higher = [](double x, double y) { return less64(x, y) ? y : x; };
   const double rL = uL[0], rR = uR[0];
   const double iL = 1.0 / (rL), iR = 1.0 / (rR);
   double vL[D], vR[D], unL = 0, unR = 0, kL = 0, kR = 0;
@@ -81,8 +89,8 @@ __device__ __forceinline__ void hllc64(const double *uL, const double *uR, const
   }
   const double Ht = (HL + HR * Dr) * idn;
   const double ct = sqrt64((g - 1) * (Ht - 0.5 * ut2));
-  const double SL = lower(unL - cL, utn - ct);
-  const double SR = higher(unR + cR, utn + ct);
+  const double SL = lower64(unL - cL, utn - ct);
+  const double SR = higher64(unR + cR, utn + ct);
   const double SM = quotient(rR * unR * (SR - unR) - rL * unL * (SL - unL) + pL - pR,
                        rR * (SR - unR) - rL * (SL - unL));
   // The four cases, tested in the order SL > 0 (left state), SM > 0 (left star state), SR > 0
