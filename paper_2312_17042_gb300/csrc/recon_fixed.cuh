@@ -263,7 +263,8 @@ __global__ void __launch_bounds__(128, TileShape<D, R, 8>::BLOCKS) recon_fixed_k
   // where the range is so small that the high words overestimate it by more than 2^-8, from the whole means: the
   // decisions depend on ratios of indicators, so the differences need their own relative accuracy
   const int eu = (max(kmax, ~kmin) >> 20) & 0x7FF;
-  if (__any_sync(0xffffffffu, ((__double2hiint(range) >> 20) & 0x7FF) < eu - 12)) {
+  const bool near = ((__double2hiint(range) >> 20) & 0x7FF) < eu - 12;
+  if (__any_sync(0xffffffffu, near)) {
     auto key64 = [](double u) {
       const long long b = __double_as_longlong(u);
       return b ^ ((b >> 63) & 0x7FFFFFFFFFFFFFFFll);
@@ -281,7 +282,7 @@ __global__ void __launch_bounds__(128, TileShape<D, R, 8>::BLOCKS) recon_fixed_k
       }
     }
     auto value = [](long long k) { return __longlong_as_double(k ^ ((k >> 63) & 0x7FFFFFFFFFFFFFFFll)); };
-    range = value(lmax) - value(lmin);
+    if (near) range = value(lmax) - value(lmin);  // a lane's unit depends on its own stencil only
   }
   const int er = max((__double2hiint(range) >> 20) & 0x7FF, 64);  // |U_m - U_0| < 2^(er - 1022)
   // a non-finite member makes every coefficient NaN

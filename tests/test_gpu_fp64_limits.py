@@ -71,3 +71,36 @@ def test_cut_off_that_drops_every_stencil(name, guard):
     assert (o.flags() == 0).any()
     assert np.array_equal(flags, o.flags()) and count.value == o.nguard()
     assert _relerr(got.reshape(-1, d + 2).T, o.face_states().reshape(-1, d + 2).T) < 1e-12
+
+
+@pytest.mark.parametrize("name", list(MESHES))
+def test_face_states_do_not_depend_on_the_cells_of_the_warp(name):
+    """A mesh alone and as the second of a batch, whose first cells share a warp with the last ones of the first: the
+    same bits. The first mesh is uniform, so that the range of its stencils is taken again from the whole means. The
+    momenta of the second reach from -1 to 1 - 2^-40 in most stencils: the bound of that range by the high words is
+    in the next binade, and the unit of the differences would be another. C_T = 0 keeps the central stencil."""
+    native = _native()
+    make, degree = MESHES[name]
+    wl = make()
+    d, n = wl.mesh.dim, wl.mesh.ncells
+    small = {"tri-r2": lambda: W.shock_tube_2d(5, 9), "tri-r5": lambda: W.shock_tube_2d(9, 5),
+             "tet-r3": lambda: _ragged(W.blast_3d(4), 1), "tet-r2": lambda: _ragged(W.density_wave_3d(4), 1)}
+    first = small.get(name, lambda: W.density_wave_2d(13))()
+    assert first.mesh.ncells % (8 if d == 2 else 6)
+    flat = np.repeat(np.array([1.0] + [0.5, -0.25, 0.125][:d] + [2.0])[:, None], first.mesh.ncells, axis=1)
+    for seed in range(3):
+        rng = np.random.default_rng(seed)
+        U = rng.uniform(1, 2, (d + 2, n))
+        U[1:-1] = rng.uniform(-0.9, 0.9, (d, n))
+        pick = rng.integers(0, 4, (d, n))
+        U[1:-1][pick == 0] = -1.0
+        U[1:-1][pick == 1] = 1.0 - 2.0 ** -40
+        out = []
+        for meshes, states in (([wl.mesh], [U]), ([first.mesh, wl.mesh], [flat, U])):
+            s = _solver(native, meshes, d, degree=degree, C_T=0.0, positivity_guard=0)
+            for k, u in enumerate(states):
+                s.set_state(u, k)
+            s.stage(0, 0.0)
+            out.append(native.cteno_get_face_states(s.ctx, len(meshes) - 1))
+            s.close()
+        assert np.array_equal(out[0], out[1])
