@@ -75,8 +75,9 @@ typedef struct {
                            stencil with the weights of eq. 14, b = 4, on the CWENO split p_1) and
                            CTENO_SCHEME_TENO (Sec. 2.4: the cut-off of eqs. 19-23 without linear
                            coefficients, on the central least-squares polynomial itself) */
-  int precision;        /* CTENO_FP64: FP64 throughout (the inner products of the conserved-variable
-                           reconstruction as sums of 57-bit block fixed-point integers). CTENO_MIXED:
+  int precision;        /* CTENO_FP64: FP64 throughout (the central inner products of the conserved-variable
+                           reconstruction as sums of 57-bit block fixed-point integers: accurate to
+                           the rounding of the largest mean of the central stencil). CTENO_MIXED:
                            reconstruction and flux in FP32; geometry, least-squares build, residual
                            accumulation and the RK update in FP64 */
   int lam_gamma;        /* 1: scale-separation measure gamma_s carries the linear coefficient

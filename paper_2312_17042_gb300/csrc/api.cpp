@@ -44,7 +44,7 @@ struct cteno_ctx {
   int hrec = 0, hms = 0;
   uint32_t *cinfo = nullptr, *fmeta = nullptr;
   void *Pc = nullptr, *Pd = nullptr, *Uf = nullptr;
-  int8_t *Pe = nullptr;              // FP64 path, conserved variables: block exponents of Pc, Pd
+  int8_t *Pe = nullptr;              // FP64 path, conserved variables: block exponents of Pc
   int32_t *phifx = nullptr;          //   and the face table
   uint8_t *flags = nullptr;
   double *geo = nullptr, *vol = nullptr, *dt = nullptr;

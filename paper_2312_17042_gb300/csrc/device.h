@@ -81,9 +81,9 @@ struct DevTables {
 //   Pc      T      [N][M][nk]      central pseudo-inverse, member-major; in tiles (tiles.h) on the FP64
 //                                  path and at degrees 4 to 6, conserved variables
 //   Pd      T      [N][NF][PDS]    directional pseudo-inverses (layout of Dir<D, R>)
-//           FP64 path, conserved variables: Pc and Pd hold int2 (h, l), entries of 57-bit integers
-//           (layout in tiles.h)
-//   Pe      int8   [N][kFixExp]    block exponents of those: rows of Pc, then faces of Pd
+//           FP64 path, conserved variables: Pc holds int2 (h, l), entries of 57-bit integers
+//           (layouts in tiles.h)
+//   Pe      int8   [N][kFixExp]    their block exponents, one per row
 //   Uf      T      [N][NF][NQ][NV] face Gauss-point states
 //   nbr     int32  [N][4]          face neighbours, -1 on a boundary
 //   geo     double [N][NF][4]      outward unit normal (n_x, n_y[, n_z]) and area in slot 3;
@@ -175,7 +175,7 @@ struct SetupArgs {
   void *Pc, *Pd;            // outputs, T = double (FP64 path) or float (mixed path)
   int store_fp32;
   int tiled;                // Pc in the layout of tiles.h
-  int8_t *Pe;               // not null: Pc, Pd as 57-bit integers, Pe their exponents
+  int8_t *Pe;               // not null: Pc as 57-bit integers, Pe their exponents (FP64 path)
   double *geo, *vol;       // vol receives 1 / |V_i|
   float *geo32;
   const DevTables *tab;

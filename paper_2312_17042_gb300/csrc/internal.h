@@ -19,7 +19,7 @@ constexpr int kMaxNQ = 4;    // Gauss points per face (3D; 2D degree 6)
 constexpr int kMaxNV = 5;    // conserved variables in 3D
 constexpr int kMaxDir = 10;  // members of a directional stencil (2d; 10 for the quadratic ones)
 constexpr int kMaxPerm = 6;  // orderings of a face's vertices
-constexpr int kFixExp = 32;  // bytes of a cell's block exponents (FP64 path): K-1 rows, then the faces
+constexpr int kFixExp = 32;  // bytes of a cell's block exponents (FP64 path): K-1 rows
 constexpr int kMaxVQ = 16;   // points of the volume rule (4 x 4 in 2D at degree 6)
 
 // K(r,d) of eq. 6: number of monomials of degree <= r in d variables, constant included.

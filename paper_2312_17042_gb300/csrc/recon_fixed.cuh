@@ -3,13 +3,13 @@
 //
 // The FP64 pipe of this GPU retires about 2 lanes per clock and SM, the integer multiply-add
 // (32 x 32 + 64 bits) 60: an inner product of 57-bit integers costs three of those, a tenth of the
-// FP64 time. The products with the least-squares operators and with the face-point basis are
+// FP64 time. The products with the central least-squares operators and with the face-point basis are
 // therefore taken over block fixed-point numbers: both factors are integers of 57 bits and a sign
 // relative to the largest of their block, x = h 2^29 + l with |h| <= 2^28, |l| <= 2^28, and
 //   sum x y = 2^58 sum h h' + 2^29 sum (h l' + l h') + sum l l',
 // whose first two sums fit 64-bit accumulators exactly for up to 56 terms. The last one, below
 // 2^-58 of the block maxima per term, is dropped: an FP64 product rounds at 2^-53 of itself.
-//   operators   per row (unknown) of a cell, scaled by the set-up kernel to the row's largest entry;
+//   operators   the central ones, per row (unknown) of a cell, scaled by the set-up kernel to the row's largest entry;
 //   U_m - U_0   exact differences of the FP64 means (modulo 2^64) in units of 2^-57 of a bound of the
 //               variable's range over the stencil, which a first pass takes from the high words;
 //   face values the coefficients against the largest |a_k| max|phi_k|, the table per basis function.
@@ -17,18 +17,26 @@
 // phi' = L^-1 phi, folded into the operators at set-up), so that an indicator (eq. 15) is a sum of K-1
 // squares instead of (K-1)(K+2)/2 products. p_1 and U_0 + p stay FP64.
 //
+// The directional products stay FP64 too. A cell beside a jump drops the central stencil and keeps directional
+// ones on its own side, whose differences may be any fraction of the central stencil's range: in its unit they
+// lost their last places, 3e-11 of the low side's means at a jump of 1e6 and 3e-7 at 1e10 (2D degree 3; now 2e-16 at
+// both, as without a jump). Where the central polynomial is kept, its values are three times as close to exact sums as
+// FP64 products are, of the largest mean of the stencil (at most three times as far, still 1e-16 of it, if only the
+// stencil's least weighted member is across a jump). In FP64 they cost 0 to 4 us a launch of those below, most at
+// degree 5, where each of the 150 products takes the pipe for 64 clocks of a lone warp.
+//
 // The selection (eqs. 19-23) and the positivity test only yield decisions: they are taken in FP32
 // where they hold by a margin far above its error, and in FP64 as printed elsewhere.
 //
 // Schedule: variable per lane, as recon_lane, one tile per warp. The operators stream through the warp's
 // ring of shared-memory stages, one bulk copy per chunk (tiles.h), issued before the previous kernel has
 // ended: read from global memory they cost twice the time, at 8 to 16 warps per SM. The
-// differences of the directional members (the first slots of the stencil list) wait in shared
+// FP64 differences of the directional members (the first slots of the stencil list) wait in shared
 // memory between the two products.
 //
 // Measured per launch against the FP64 schedules it replaced (bound by the FP64 pipe, 61 to 86 % of its
-// rate): 2D degree 3, 131 072 cells 534 -> 120 us; 3D degree 3, 24 576 cells 432 (553 in blocks of 128) -> 133
-// us; 2D degree 5, 4200 cells 81 -> 36 us; 2D degree 2, 2048 cells 19 (51 in blocks of 128) -> 12 us. It is
+// rate): 2D degree 3, 131 072 cells 534 -> 121 us; 3D degree 3, 24 576 cells 432 (553 in blocks of 128) -> 127
+// us; 2D degree 5, 4200 cells 81 -> 41 us; 2D degree 2, 2048 cells 19 (51 in blocks of 128) -> 11 us. It is
 // now bound by the integer pipe (shifts and 64-bit sums of the conversions, 63 % busy at 2D degree 3), the
 // small meshes by the length of a warp's chain.
 #pragma once
@@ -170,7 +178,7 @@ __global__ void __launch_bounds__(128, TileShape<D, R, 8>::BLOCKS) recon_fixed_k
   const int4 *const sPhi = reinterpret_cast<const int4 *>(smem);
   uint64_t *const tbar = reinterpret_cast<uint64_t *>(smem + S::PHI_BYTES);  // the block's: face table
   unsigned char *const wmem = smem + S::PHI_BYTES + 16 + (threadIdx.x >> 5) * S::WARP_BYTES;
-  int2 *const sdel = reinterpret_cast<int2 *>(wmem + S::HDR + NST * S::STAGE) + (threadIdx.x & 31);
+  double *const sdel = reinterpret_cast<double *>(wmem + S::HDR + NST * S::STAGE) + (threadIdx.x & 31);
   uint64_t *const bar = reinterpret_cast<uint64_t *>(wmem + S::HDR + NST * S::STAGE + S::DELTA);  // header, stages
   const int lane = threadIdx.x & 31, grp = lane / NV, v = lane - grp * NV, base = grp * NV;
   const int64_t N = a.N;
@@ -194,7 +202,7 @@ __global__ void __launch_bounds__(128, TileShape<D, R, 8>::BLOCKS) recon_fixed_k
     if (n > 0) {
       mbar_arrive_expect_tx(&bar[0], (uint32_t)(CPW * M * 4 + n * NF * PDS * 8));
       bulk_copy_g2s(wmem + S::HPD, a.st + c0 * M, (uint32_t)(CPW * M * 4), &bar[0]);
-      bulk_copy_g2s(wmem, (const int2 *)a.Pd + c0 * (NF * PDS), (uint32_t)(n * NF * PDS * 8), &bar[0]);
+      bulk_copy_g2s(wmem, (const double *)a.Pd + c0 * (NF * PDS), (uint32_t)(n * NF * PDS * 8), &bar[0]);
       for (int c = 0; c < NST; ++c) issue(c);
     }
   }
@@ -285,7 +293,7 @@ __global__ void __launch_bounds__(128, TileShape<D, R, 8>::BLOCKS) recon_fixed_k
     if (near) range = value(lmax) - value(lmin);  // a lane's unit depends on its own stencil only
   }
   const int er = max((__double2hiint(range) >> 20) & 0x7FF, 64);  // |U_m - U_0| < 2^(er - 1022)
-  // a non-finite member makes every coefficient NaN
+  // a non-finite member makes every central coefficient NaN
   const bool finite = kmax < 0x7FF00000 && kmin > (int)0x800FFFFF && er < 0x7FF;
   const int64_t F0 = fx_of(U0, er, 1 << 28);
 
@@ -310,7 +318,7 @@ __global__ void __launch_bounds__(128, TileShape<D, R, 8>::BLOCKS) recon_fixed_k
 #pragma unroll
       for (int g = 0; g < G; ++g) {
         dx[g] = fx_split(fx_of(un[g], er, F0));
-        if (m + g < SLOTS) sdel[(m + g) * 32] = dx[g];
+        if (m + g < SLOTS) sdel[(m + g) * 32] = un[g] - U0;
       }
       if (m + G < M) {
         int j[G];
@@ -348,7 +356,7 @@ __global__ void __launch_bounds__(128, TileShape<D, R, 8>::BLOCKS) recon_fixed_k
   }
   // directional coefficients: the members of face f are the next slots of the list
   const uint32_t adm = (info >> kInfoAdmShift) & 0xFu;
-  const int2 *__restrict__ Pdi = reinterpret_cast<const int2 *>(wmem) + slot * (NF * PDS);
+  const double *__restrict__ Pdi = reinterpret_cast<const double *>(wmem) + slot * (NF * PDS);
   double ad[NF][KD];
   {
     int off = 0;
@@ -358,42 +366,26 @@ __global__ void __launch_bounds__(128, TileShape<D, R, 8>::BLOCKS) recon_fixed_k
 #pragma unroll
       for (int k = 0; k < KD; ++k) ad[f][k] = 0.0;
       if ((adm >> f) & 1u) {
-        int64_t A1[KD], A2[KD];
-#pragma unroll
-        for (int k = 0; k < KD; ++k) A1[k] = A2[k] = 0;
 #pragma unroll
         for (int jj = 0; jj < ND; jj += 2) {
-          if (jj < nm) {  // an odd last member is followed by zero entries of the operator
-            const int2 d0 = sdel[(off + jj) * 32], d1 = sdel[min(off + jj + 1, SLOTS - 1) * 32];
+          if (jj < nm) {
+            const double d0 = sdel[(off + jj) * 32], d1 = jj + 1 < nm ? sdel[(off + jj + 1) * 32] : 0.0;
 #pragma unroll
             for (int c = 0; c < KD; ++c) {
-              const int4 p = reinterpret_cast<const int4 *>(Pdi + f * PDS + jj * KD)[c];
-              const int ph[2] = {p.x, p.z}, pl[2] = {p.y, p.w};
-#pragma unroll
-              for (int t = 0; t < 2; ++t) {
-                const int k = (2 * c + t) % KD;
-                const int2 dx = (2 * c + t) / KD ? d1 : d0;
-                fx_mac(A1[k], ph[t], dx.x);
-                fx_mac(A2[k], ph[t], dx.y);
-                fx_mac(A2[k], pl[t], dx.x);
-              }
+              const double2 p = reinterpret_cast<const double2 *>(Pdi + f * PDS + jj * KD)[c];
+              const int k = (2 * c) % KD, l = (2 * c + 1) % KD;
+              ad[f][k] = fma(p.x, 2 * c / KD ? d1 : d0, ad[f][k]);
+              ad[f][l] = fma(p.y, (2 * c + 1) / KD ? d1 : d0, ad[f][l]);
             }
           }
         }
-#pragma unroll
-        for (int k = 0; k < KD; ++k) ad[f][k] = fx_to_double(A1[k], A2[k], 29 - 57 - 1079 + er + __ldg(ei + NK + f));
       }
       off += nm;
     }
   }
   if (!finite) {
-    const double bad = __longlong_as_double(0x7FF8000000000000ll);
 #pragma unroll
-    for (int k = 0; k < NK; ++k) ao[k] = bad;
-#pragma unroll
-    for (int f = 0; f < NF; ++f)
-#pragma unroll
-      for (int k = 0; k < KD; ++k) ad[f][k] = ((adm >> f) & 1u) ? bad : 0.0;
+    for (int k = 0; k < NK; ++k) ao[k] = __longlong_as_double(0x7FF8000000000000ll);
   }
 
   // p_1 (eq. 17) without its factor 1 / lambda_1, which goes to the face values (`scale`)

@@ -263,19 +263,14 @@ __global__ void __launch_bounds__(128) setup_kernel(const SetupArgs a) {
       }
     }
     constexpr int PDS = DR::PDS;
-    if (a.Pe) {  // FP64 path: orthonormal basis, 57-bit integers, member-major
-      double top = 0.0;
-      for (int j = 0; j < ND; ++j)
-        for (int k = 0; k < KD; ++k) {
-          double s = 0.0;
+    if (a.Pe) {  // FP64 path, conserved variables: orthonormal basis, member-major
+      for (int t = 0; t < PDS; ++t) {
+        const int j = t / KD, k = t % KD;
+        double s = 0.0;
+        if (j < ND)
           for (int l = k; l < KD; ++l) s += T.LT[k][l] * pd[l][j];
-          pd[k][j] = s;
-          top = fmax(top, fabs(s));
-        }
-      const int e = block_exponent(top);
-      a.Pe[i * kFixExp + NK + f] = (int8_t)e;
-      for (int t = 0; t < PDS; ++t)
-        ((int2 *)a.Pd)[(i * NF + f) * PDS + t] = (t < ND * KD) ? to_fixed(pd[t % KD][t / KD], e) : make_int2(0, 0);
+        ((double *)a.Pd)[(i * NF + f) * PDS + t] = s;
+      }
       off += nm;
       continue;
     }

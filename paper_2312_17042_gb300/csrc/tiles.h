@@ -5,8 +5,8 @@
 // central rows in chunks of MC members, so that the chunk a warp copies is one contiguous span:
 //   Pc  [tile][M / MC][CPW][MC][NK]   (the last tile is allocated whole)
 //   Pd  [cell][face][PDS]             (Dir<D, R>; FP64 path: member-major j * KD + k at every degree)
-// Entries (E bytes): float, or on the FP64 path int2 (h, l), the integer h 2^29 + l of 57 bits and a
-// sign in units of 2^(e - 57), e the exponent of its block (KArgs::Pe).
+// Entries (E bytes): float, or on the FP64 path Pd double and Pc int2 (h, l), the integer h 2^29 + l of 57 bits
+// and a sign in units of 2^(e - 57), e the exponent of its row (KArgs::Pe).
 #pragma once
 
 #include <cstdint>

@@ -23,6 +23,47 @@ MESHES = {
 }
 
 
+@pytest.mark.parametrize("jump", [1e2, 1e6, 1e10])
+@pytest.mark.parametrize("scheme", [0, 1, 3], ids=["CTENO", "CTENOZ-wenoz", "TENO"])
+@pytest.mark.parametrize("name", list(MESHES))
+def test_low_side_of_a_jump(name, scheme, jump):
+    """A jump of all variables between two smooth states: the cells beside it drop the stencils that cross it, and
+    their face states are as accurate as products in FP64 give them, of the largest |U_v| over the members of the
+    stencils that are kept (1e-12; max(1e-12, 50 cond(A) u) at degrees 4 to 6)."""
+    native = _native()
+    from oracle import Oracle
+    make, degree = MESHES[name]
+    wl = make()
+    d, n = wl.mesh.dim, wl.mesh.ncells
+    x = W.cell_centroids(wl.mesh)
+    t = (x - x.min(0)) / np.ptp(x, axis=0).max()
+    wave = 1 + 0.1 * np.sin(3 * t @ np.array([1.0, 0.7, 0.4])[:d] + np.arange(d + 2)[:, None])
+    U = np.array([1.0] + [0.3, -0.2, 0.1][:d] + [2.5])[:, None] * wave * np.where(t[:, 0] > 0.5 * t[:, 0].max(), jump, 1.0)
+    o = Oracle(wl.mesh, degree=degree, scheme=scheme, ctenoz_form=1)
+    tol = 1e-12
+    if degree >= 4:
+        tol = max(tol, 50 * max(np.linalg.cond(o.lsq(i)[0]) for i in range(0, n, max(1, n // 60))) * 2.0 ** -53)
+    o.set_state(U)
+    o.residual()
+    s = _solver(native, [wl.mesh], d, degree=degree, scheme=scheme, ctenoz_form=1)
+    native.cteno_record_flags(s.ctx, True)
+    s.set_state(U)
+    s.stage(0, 0.0)
+    got, flags = native.cteno_get_face_states(s.ctx, 0), native.cteno_get_flags(s.ctx, 0)
+    s.close()
+    assert np.array_equal(flags, o.flags())
+    scale = np.abs(U)
+    for i in range(n):
+        central, directional, ok = o.stencil(i)
+        for v in range(d + 2):
+            kept = [central] if flags[i, v] & 1 else \
+                [directional[f][directional[f] >= 0] for f in range(d + 1) if flags[i, v] >> (1 + f) & 1]
+            scale[v, i] = max([scale[v, i]] + [np.abs(U[v, m]).max() for m in kept])
+    low = t[:, 0] <= 0.5 * t[:, 0].max()
+    assert (scale[0, low] < 2).any() and (flags[low, 0] & 1 == 0).any()
+    assert np.all(np.abs(got - o.face_states()).reshape(n, -1, d + 2) <= tol * scale.T[:, None])
+
+
 @pytest.mark.parametrize("guard", [0, 1])
 @pytest.mark.parametrize("dim", [2, 3])
 def test_negative_pressure_on_one_side_of_a_face(dim, guard):
