@@ -331,9 +331,10 @@ int cteno_last_kernel_ms(cteno_ctx *ctx, double *ms_out);
 int cteno_measure_alu_peak(double *fp64_tflops, double *fp32_tflops);
 
 /* Test hook of the failure path of the bounded waits (no counterpart in the paper). With
- * limit_ns > 0 every launch of a staged reconstruction schedule (launch values 2048 + b, 3072 + b,
- * 4096, 4097) first waits, for at most limit_ns nanoseconds, on a shared-memory barrier that nothing
- * completes. The wait runs out: the kernel records the timeout in the context's error word, waits
+ * limit_ns > 0 every launch of a reconstruction that waits for bulk copies (FP64 and degrees 4 to 6 of
+ * the conserved variables; on the mixed path every schedule at degrees 2 and 3 but b, -b and 1024 + b)
+ * first waits, for at most limit_ns nanoseconds, on a shared-memory barrier that nothing completes; the
+ * other launches have no wait that could run out and ignore it. The wait runs out: the kernel records the timeout in the context's error word, waits
  * (bounded) for the bulk copies it has issued, and returns; the next synchronising call returns
  * CTENO_ERR_DEVICE, as for a bulk copy that never completes. 0 (the default) turns it off; limit_ns
  * is at most 1e9. The error word of the context stays set: use a new context afterwards. */

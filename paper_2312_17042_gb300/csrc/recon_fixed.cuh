@@ -179,7 +179,7 @@ __global__ void __launch_bounds__(128, TileShape<D, R, 8>::BLOCKS) recon_fixed_k
   uint64_t *const tbar = reinterpret_cast<uint64_t *>(smem + S::PHI_BYTES);  // the block's: face table
   unsigned char *const wmem = smem + S::PHI_BYTES + 16 + (threadIdx.x >> 5) * S::WARP_BYTES;
   double *const sdel = reinterpret_cast<double *>(wmem + S::HDR + NST * S::STAGE) + (threadIdx.x & 31);
-  uint64_t *const bar = reinterpret_cast<uint64_t *>(wmem + S::HDR + NST * S::STAGE + S::DELTA);  // header, stages
+  uint64_t *const bar = reinterpret_cast<uint64_t *>(wmem + S::HDR + NST * S::STAGE + S::DELTA);  // header, stages, test hook
   const int lane = threadIdx.x & 31, grp = lane / NV, v = lane - grp * NV, base = grp * NV;
   const int64_t N = a.N;
   const int64_t tile = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), c0 = tile * CPW;
@@ -192,7 +192,7 @@ __global__ void __launch_bounds__(128, TileShape<D, R, 8>::BLOCKS) recon_fixed_k
   };
   // the operators do not depend on the previous kernel: their copies start here
   if (lane == 0) {
-    for (int b = 0; b < 1 + NST; ++b) mbar_init(&bar[b], 1);
+    for (int b = 0; b < 2 + NST; ++b) mbar_init(&bar[b], 1);
     if (threadIdx.x == 0) mbar_init(tbar, 1);
     fence_barrier_init();
     if (S::PHI_BYTES && threadIdx.x == 0) {
@@ -220,8 +220,8 @@ __global__ void __launch_bounds__(128, TileShape<D, R, 8>::BLOCKS) recon_fixed_k
     }
   // a bounded wait of the whole warp for its copies; on a timeout the warp reports it, gives the
   // copies in flight (chunks c up to `last`) a second bounded wait and stops
-  auto arrived = [&](uint64_t *b, uint32_t parity, int c, int last) {
-    const bool ok = mbar_wait(b, parity, kStageWaitNs);
+  auto arrived = [&](uint64_t *b, uint32_t parity, int c, int last, uint64_t limit_ns = kStageWaitNs) {
+    const bool ok = mbar_wait(b, parity, limit_ns);
     if (!__any_sync(0xffffffffu, !ok)) return true;
     if (lane == 0) {
       atomicOr(a.err, kErrTimeout);
@@ -236,6 +236,8 @@ __global__ void __launch_bounds__(128, TileShape<D, R, 8>::BLOCKS) recon_fixed_k
     if (S::PHI_BYTES) arrived(tbar, 0, 0, 0);
     return;
   }
+  // test hook: a bounded wait on a barrier that nothing completes runs out
+  if (a.test_wait_ns && !arrived(&bar[1 + NST], 0, 0, NST, a.test_wait_ns)) return;
   const double *__restrict__ Uv = after_wait(a.U) + v;
   const int32_t *__restrict__ sti = reinterpret_cast<const int32_t *>(wmem + S::HPD) + slot * M;
   const double U0 = __ldg(Uv + i * NVP);

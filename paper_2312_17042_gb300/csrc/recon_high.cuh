@@ -239,7 +239,7 @@ __global__ void __launch_bounds__(128, TileShape<2, R, 4>::BLOCKS) recon_high_st
   extern __shared__ __align__(128) unsigned char smem[];
   unsigned char *const wmem = smem + (threadIdx.x >> 5) * S::WARP_BYTES;
   float *const sdel = reinterpret_cast<float *>(wmem + S::HDR + NST * S::STAGE) + (threadIdx.x & 31);
-  uint64_t *const bar = reinterpret_cast<uint64_t *>(wmem + S::HDR + NST * S::STAGE + S::DELTA);  // header, stages
+  uint64_t *const bar = reinterpret_cast<uint64_t *>(wmem + S::HDR + NST * S::STAGE + S::DELTA);  // header, stages, test hook
   const int lane = threadIdx.x & 31, grp = lane / NV, v = lane - grp * NV, base = grp * NV;
   const int64_t N = a.N;
   const int64_t tile = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), c0 = tile * S::CPW;
@@ -251,7 +251,7 @@ __global__ void __launch_bounds__(128, TileShape<2, R, 4>::BLOCKS) recon_high_st
                   S::STAGE, b);
   };
   if (lane == 0 && n > 0) {
-    for (int b = 0; b < 1 + NST; ++b) mbar_init(&bar[b], 1);
+    for (int b = 0; b < 2 + NST; ++b) mbar_init(&bar[b], 1);
     fence_barrier_init();
     mbar_arrive_expect_tx(&bar[0], (uint32_t)(S::CPW * M * 4 + n * NF * PDS * 4));
     bulk_copy_g2s(wmem + S::HPD, a.st + c0 * M, (uint32_t)(S::CPW * M * 4), &bar[0]);
@@ -272,8 +272,8 @@ __global__ void __launch_bounds__(128, TileShape<2, R, 4>::BLOCKS) recon_high_st
   if (n == 0) return;  // a warp past the last cell
   // a bounded wait of the whole warp for its copies; on a timeout the warp reports it, gives the
   // copies in flight (chunks c up to `last`) a second bounded wait and stops
-  auto arrived = [&](uint64_t *b, uint32_t parity, int c, int last) {
-    const bool ok = mbar_wait(b, parity, kStageWaitNs);
+  auto arrived = [&](uint64_t *b, uint32_t parity, int c, int last, uint64_t limit_ns = kStageWaitNs) {
+    const bool ok = mbar_wait(b, parity, limit_ns);
     if (!__any_sync(0xffffffffu, !ok)) return true;
     if (lane == 0) {
       atomicOr(a.err, kErrTimeout);
@@ -283,6 +283,8 @@ __global__ void __launch_bounds__(128, TileShape<2, R, 4>::BLOCKS) recon_high_st
     __syncwarp();
     return false;
   };
+  // test hook: a bounded wait on a barrier that nothing completes runs out
+  if (a.test_wait_ns && !arrived(&bar[1 + NST], 0, 0, NST, a.test_wait_ns)) return;
   const float2 *__restrict__ Uv = reinterpret_cast<const float2 *>(after_wait(a.U32)) + v;
   const int32_t *__restrict__ sti = reinterpret_cast<const int32_t *>(wmem + S::HPD) + slot * M;
   const float2 own = __ldg(Uv + i * NVP);

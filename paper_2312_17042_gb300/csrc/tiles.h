@@ -42,7 +42,7 @@ struct TileShape {
   static constexpr int STAGE = CPW * MC * NK * E;
   // a warp's header: directional operators, then stencil ids
   static constexpr int HPD = CPW * NF * PDS * E, HDR = HPD + CPW * M * 4, DELTA = SLOTS * 32 * E;
-  static constexpr int BARS = (1 + NST + 1) / 2 * 16;
+  static constexpr int BARS = (2 + NST + 1) / 2 * 16;  // header, stages, test hook
   static constexpr int WARP_BYTES = HDR + NST * STAGE + DELTA + BARS;
   __host__ __device__ static constexpr int64_t index(int64_t cell, int m, int k) {  // of entry (m, k) of a cell in Pc
     const int64_t t = cell / CPW;
