@@ -6,7 +6,7 @@
 // the mesh gives:
 //   face_flux64    one lane per face Gauss point (not per face): HLLC once per face in its owner's
 //                  orientation, comparisons and selections on integers, square roots from the hardware estimate
-//                  and two corrections; the points of a face are exchanged by shuffles and summed in order;
+//                  (sqrt64.cuh); the points of a face are exchanged by shuffles and summed in order;
 //   cell_update64  one lane per conserved variable: the cell's face fluxes, signed, in face order,
 //                  the Runge-Kutta update and, over the same lanes, the CFL step.
 // The per-cell schedules of the mixed path evaluate every face twice; in FP64 they took three times
@@ -19,21 +19,11 @@
 // of 32 threads, 20.4 in blocks of 128), large ones do not care (146.7 / 146.3 us): 32 by default.
 #pragma once
 
+#include "sqrt64.cuh"
+
 namespace cteno {
 namespace {
 
-// sqrt(x): coupled iteration on g ~ sqrt(x) and h ~ 1 / (2 sqrt(x)) (Goldschmidt), then the
-// residual correction g + (x - g^2) h. Values below the normal numbers give 0.
-__device__ __forceinline__ double sqrt64(const double x) {
-  double y;
-  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-  double g = x * y, h = __hiloint2double(__double2hiint(y) - (1 << 20), __double2loint(y));  // y / 2
-  const double r = fma(-g, h, 0.5);
-  g = fma(g, r, g);
-  h = fma(h, r, h);
-  g = fma(fma(-g, g, x), h, g);
-  return (__double2hiint(x) & 0x7FFFFFFF) < 0x00100000 ? 0.0 : g;
-}
 // x > 0, and fmin(a, b), fmax(a, b) with their rule for NaN (the other operand: a side with a negative pressure has
 // no speed of sound, and the wave speeds are then those of the other side and of the Roe average), on integers.
 __device__ __forceinline__ bool positive64(const double x) {
