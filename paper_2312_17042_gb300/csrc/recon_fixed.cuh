@@ -13,6 +13,7 @@
 //   U_m - U_0   exact differences of the FP64 means (modulo 2^64) in units of 2^-57 of a bound of the
 //               variable's range over the stencil, which a first pass takes from the high words;
 //   face values the coefficients against the largest |a_k| max|phi_k|, the table per basis function.
+// Ranges and coefficients keep their places from 2^-950 on, lose them one by one below and are zero below 2^-1007.
 // The coefficients are those of a basis orthonormal in the smoothness form (O = L L^T, b = L^T a,
 // phi' = L^-1 phi, folded into the operators at set-up), so that an indicator (eq. 15) is a sum of K-1
 // squares instead of (K-1)(K+2)/2 products. p_1 and U_0 + p stay FP64.
@@ -297,6 +298,9 @@ __global__ void __launch_bounds__(128, TileShape<D, R, 8>::BLOCKS) recon_fixed_k
   const int er = max((__double2hiint(range) >> 20) & 0x7FF, 64);  // |U_m - U_0| < 2^(er - 1022)
   // a non-finite member makes every central coefficient NaN
   const bool finite = kmax < 0x7FF00000 && kmin > (int)0x800FFFFF && er < 0x7FF;
+  // means near the largest numbers: central coefficients in units of 2^200, taken back by `scale`, so that what does
+  // not fit becomes infinite in a face value (the guard's case) and not zero in a coefficient
+  const bool top_range = finite && er > 1900;
   const int64_t F0 = fx_of(U0, er, 1 << 28);
 
   // central coefficients b = P_c (U_m - U_0)
@@ -354,7 +358,7 @@ __global__ void __launch_bounds__(128, TileShape<D, R, 8>::BLOCKS) recon_fixed_k
     }
     // P = h 2^29 + l in units of 2^(E_k - 57), the differences in units of 2^(er - 1079)
 #pragma unroll
-    for (int k = 0; k < NK; ++k) ao[k] = fx_to_double(A1[k], A2[k], 29 - 57 - 1079 + er + __ldg(ei + k));
+    for (int k = 0; k < NK; ++k) ao[k] = fx_to_double(A1[k], A2[k], 29 - 57 - 1079 - (top_range ? 200 : 0) + er + __ldg(ei + k));
   }
   // directional coefficients: the members of face f are the next slots of the list
   const uint32_t adm = (info >> kInfoAdmShift) & 0xFu;
@@ -394,7 +398,7 @@ __global__ void __launch_bounds__(128, TileShape<D, R, 8>::BLOCKS) recon_fixed_k
   const int stn = 1 + __popc(adm);
   const bool split = stn > 1 && a.central_split;
   if (split) {
-    const double lams = pick<NF>(a.lams_d, stn - 1);
+    const double lams = pick<NF>(a.lams_d, stn - 1) * (top_range ? 0x1p-200 : 1.0);
 #pragma unroll
     for (int k = 0; k < KD; ++k) {
       double s = ad[0][k];
@@ -404,10 +408,11 @@ __global__ void __launch_bounds__(128, TileShape<D, R, 8>::BLOCKS) recon_fixed_k
     }
   }
   double scale = split ? a.inv_lam1 : 1.0;
+  if (top_range) scale *= 0x1p200;
   // the indicators (eq. 15) and the selection (eqs. 19-23) or the weights (eq. 14)
   uint32_t bits = 0u;
   bool sure = false;
-  if (!a.cweno) {
+  if (!a.cweno && !top_range) {
     float s0 = 0.0f, sd[NF];
 #pragma unroll
     for (int k = 0; k < NK; ++k) {
@@ -468,8 +473,9 @@ __global__ void __launch_bounds__(128, TileShape<D, R, 8>::BLOCKS) recon_fixed_k
   }
   if (a.flags && active) a.flags[v * N + i] = (uint8_t)bits;
 
-  // face values U_0 + sum_k b_k phi'_k: the coefficients in units of the largest |b_k| max |phi'_k|
-  int ef = 128;
+  // face values U_0 + sum_k b_k phi'_k: the coefficients in units of the largest |b_k| max |phi'_k|, which keep all
+  // their places from 2^-950 on (phi_exp is 1 at most)
+  int ef = 72;
 #pragma unroll
   for (int k = 0; k < NK; ++k) ef = max(ef, ((__double2hiint(ao[k]) >> 20) & 0x7FF) + a.phi_exp[k]);
   bool nan = false;

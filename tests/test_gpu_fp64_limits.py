@@ -145,3 +145,39 @@ def test_face_states_do_not_depend_on_the_cells_of_the_warp(name):
             out.append(native.cteno_get_face_states(s.ctx, len(meshes) - 1))
             s.close()
         assert np.array_equal(out[0], out[1])
+
+
+@pytest.mark.parametrize("scheme", [0, 2], ids=["CTENO", "CWENO"])
+@pytest.mark.parametrize("exponent", [-930, 1015, 1021])
+@pytest.mark.parametrize("name", list(MESHES))
+def test_means_near_the_ends_of_the_exponents(name, exponent, scheme):
+    """Fluid at rest in units of 2^exponent: a cell has the face states of the same flow in units of 2^-800 or 2^900
+    (the indicators vanish against eps or overflow there too: the same selection), or, where coefficients or face
+    values do not fit the range of the numbers, it has its mean at every face, counted by the positivity guard."""
+    native = _native()
+    from oracle import Oracle
+    make, degree = MESHES[name]
+    wl = make()
+    d, n = wl.mesh.dim, wl.mesh.ncells
+    unit = -800 if exponent < 0 else 900
+    U = wl.U0 / 10
+    U[1:-1] = 0.0
+    o = Oracle(wl.mesh, degree=degree, scheme=scheme)
+    o.set_state(np.ldexp(U, unit))
+    o.residual()
+    tol = max(1e-12, 50 * max(np.linalg.cond(o.lsq(i)[0]) for i in range(0, n, max(1, n // 60))) * 2.0 ** -53)
+    s = _solver(native, [wl.mesh], d, degree=degree, scheme=scheme)
+    s.set_state(np.ldexp(U, exponent))
+    s.stage(0, 0.0)
+    got = native.cteno_get_face_states(s.ctx, 0).reshape(n, -1, d + 2)
+    count = ctypes.c_int64(-1)
+    native.load_library().cteno_sync(s.ctx, ctypes.byref(count))
+    s.close()
+    ref = o.face_states().reshape(n, -1, d + 2)
+    same = (np.abs(np.ldexp(got, -exponent) - np.ldexp(ref, -unit)) <= tol * np.abs(U).max(axis=1)).all(axis=(1, 2))
+    mean = (got == np.ldexp(U, exponent).T[:, None]).all(axis=(1, 2))
+    assert np.all(same | mean)
+    flat = (ref == np.ldexp(U, unit).T[:, None]).all(axis=(1, 2)) & ~o.guarded()
+    assert count.value == np.count_nonzero(mean & ~flat)
+    if exponent < 1015:
+        assert np.all(same)
