@@ -580,10 +580,16 @@ def run_ours(args, rank, world, local):
 
 
 def headline(result):
-    """The benchmark's one line: the measured workload in full and every variant's value. What else a variant
-    measured goes to stderr, a line each: in the line itself, some 25 kB, a reader that keeps the end of the
-    output loses the headline."""
-    return {**result, "variants": {name: v["value"] for name, v in result["variants"].items()}}
+    """The benchmark's one line: the measured workload in full and every variant's value, [mixed, fp64] per
+    workload and scheme (null where not measured). What else a variant measured goes to stderr, a line each: in
+    the line itself, some 50 kB, a reader that keeps the end of the output loses the headline."""
+    table = {}
+    for name, v in result["variants"].items():
+        workload, variant = name.split(":")
+        scheme, precision = variant.rsplit("_", 1)
+        pair = table.setdefault(workload, {}).setdefault(scheme, [None, None])
+        pair[("mixed", "fp64").index(precision)] = v["value"]
+    return {**result, "variants": table}
 
 
 def _subbox_sample(case, target):
