@@ -300,10 +300,13 @@ int cteno_sync(cteno_ctx *ctx, int64_t *guard_count);
  * most, as at degrees 4 to 6). */
 int cteno_set_launch(cteno_ctx *ctx, int recon_block, int flux_block);
 
-/* Time the candidate launch configurations (block sizes 64/128/256, on the mixed path the
- * register-capped variants at 64/128 and the staged, gather-staged and streamed reconstruction
- * schedules that fit, and the lane schedules at 128/256 threads) on the current state and keep the
- * fastest; the state is restored afterwards. The current state must be a valid one (set it first:
+/* Time the candidate launch configurations on the current state and keep the fastest; the state is
+ * restored afterwards. Mixed path, degrees 2 and 3: block sizes 64/128/256, the register-capped variants at
+ * 64/128, the lane schedules at 128/256 threads, the staged, gather-staged and streamed reconstructions that
+ * fit, and the tile-per-warp ones at 32/64/128 (in 3D these only where a lane schedule was the fastest before
+ * them, whose face values they share); degrees 4 to 6: 1024 + 32/64/128; flux: also the face-based schedule.
+ * FP64: threads per block, 64/128/256 for the reconstruction and 32/64/128 for the flux. Characteristic
+ * variables: 1024 + 64/128/256. The current state must be a valid one (set it first:
  * the kernels run on it). best_out[2] (may be NULL) receives the chosen values, in the convention
  * of cteno_set_launch. */
 int cteno_autotune(cteno_ctx *ctx, int32_t *best_out);

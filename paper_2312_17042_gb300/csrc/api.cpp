@@ -1004,7 +1004,7 @@ int cteno_set_launch(cteno_ctx *ctx, int recon_block, int flux_block) {
   auto ok = [&](int b, bool recon) {
     if (b == 0) return true;
     if (recon && ctx->p.degree >= 4) {  // degrees 4 to 6: the variable-per-lane schedule only
-      if (b >= kHighOcc + 32 && b <= kHighOcc + 256 && b % 32 == 0)  // its 64-register build
+      if (b >= kHighOcc + 32 && b <= kHighOcc + 256 && b % 32 == 0)  // the same kernel, mixed
         return ctx->fp32 && !ctx->p.characteristic;
       return b >= kLaneSchedule + 32 && b <= kLaneSchedule + 256 && b % 32 == 0;
     }
@@ -1013,7 +1013,7 @@ int cteno_set_launch(cteno_ctx *ctx, int recon_block, int flux_block) {
       return b >= kLaneSchedule + 32 && b <= kLaneSchedule + 256 && b % 32 == 0;
     if (b >= kFaceFlux && b < kTileLanes2)  // face-based flux schedule
       return !recon && b - kFaceFlux >= 32 && b - kFaceFlux <= 256 && b % 32 == 0;
-    if (tile_launch(b))  // two variables per lane: reconstruction, mixed
+    if (tile_launch(b))  // a tile per warp, one or two variables per lane: reconstruction, mixed
       return recon && ctx->fp32 && (b > kTileLanes2 || pair_fits(ctx->d, ctx->p.degree, b));
     if (b > kStreamCells && b <= kStreamCells + 8)  // streamed cells: reconstruction, mixed, fits
       return recon && ctx->fp32 &&

@@ -8,7 +8,7 @@
 //                  orientation, comparisons and selections on integers, square roots from the hardware estimate
 //                  (sqrt64.cuh); the points of a face are exchanged by shuffles and summed in order;
 //   cell_update64  one lane per conserved variable: the cell's face fluxes, signed, in face order,
-//                  the Runge-Kutta update and, over the same lanes, the CFL step.
+//                  the Runge-Kutta update and, over the same lanes, the CFL step (IEEE division and root).
 // The per-cell schedules of the mixed path evaluate every face twice; in FP64 they took three times
 // as long and are not built.
 //
@@ -44,16 +44,15 @@ __device__ __forceinline__ double higher64(const double a, const double b) {
   return (less64(b, a) || nan64(b)) && !nan64(a) ? a : b;
 }
 
-// HLLC flux as hllc() (eqs. 24-29), in its order, with IEEE division and roots to the last place: the states ahead of a
+// HLLC flux as hllc() (eqs. 24-29), in its order, with IEEE division and the roots of sqrt64: the states ahead of a
 // wave, whose selection hangs on differences of 1e-11, then round as those of any other FP64 evaluation of the
 // printed formulas does (taking common factors once and reciprocals one unit off saved a third of the time and
 // moved a 200-step shock tube by 5e-12 of its largest momentum, through selections of that size).
 template <int D>
 __device__ __forceinline__ void hllc64(const double *uL, const double *uR, const double *n, const double g, double *F) {
   constexpr int NV = D + 2;
-  auto quotient = [](double x, double y) { return x / y; };
   const double rL = uL[0], rR = uR[0];
-  const double iL = 1.0 / (rL), iR = 1.0 / (rR);
+  const double iL = 1.0 / rL, iR = 1.0 / rR;
   double vL[D], vR[D], unL = 0, unR = 0, kL = 0, kR = 0;
 #pragma unroll
   for (int j = 0; j < D; ++j) {
@@ -81,8 +80,8 @@ __device__ __forceinline__ void hllc64(const double *uL, const double *uR, const
   const double ct = sqrt64((g - 1) * (Ht - 0.5 * ut2));
   const double SL = lower64(unL - cL, utn - ct);
   const double SR = higher64(unR + cR, utn + ct);
-  const double SM = quotient(rR * unR * (SR - unR) - rL * unL * (SL - unL) + pL - pR,
-                       rR * (SR - unR) - rL * (SL - unL));
+  const double SM = (rR * unR * (SR - unR) - rL * unL * (SL - unL) + pL - pR) /
+                    (rR * (SR - unR) - rL * (SL - unL));
   // The four cases, tested in the order SL > 0 (left state), SM > 0 (left star state), SR > 0
   // (right star state), else (right state), evaluated without branches (neighbouring faces of a
   // warp take different cases): the operands of side k are selected, the star correction is

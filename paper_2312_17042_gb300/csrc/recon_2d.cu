@@ -7,7 +7,7 @@ namespace cteno {
 cudaError_t launch_recon_2d(int degree, int fp32, int scheme, const KArgs &a, int block, cudaStream_t s) {
   // the characteristic reconstruction runs in the variable-per-lane schedule only
   if (a.characteristic && !(block >= kLaneSchedule && block < kStagedCells)) return cudaErrorInvalidValue;
-  if (const int threads = tile_launch(block)) {  // two variables per lane (mixed)
+  if (const int threads = tile_launch(block)) {  // a tile per warp, one or two variables per lane (mixed)
     if (!fp32) return cudaErrorInvalidValue;  // mixed path only
     const bool one = block >= kTileLanes;
 #define CTENO_TILE(R, SC) (one ? launch_recon_tile<2, R, SC, 1>(a, threads, s) : launch_recon_tile<2, R, SC, 2>(a, threads, s))

@@ -22,9 +22,9 @@
 // ones on its own side, whose differences may be any fraction of the central stencil's range: in its unit they
 // lost their last places, 3e-11 of the low side's means at a jump of 1e6 and 3e-7 at 1e10 (2D degree 3; now 2e-16 at
 // both, as without a jump). Where the central polynomial is kept, its values are three times as close to exact sums as
-// FP64 products are, of the largest mean of the stencil (at most three times as far, still 1e-16 of it, if only the
-// stencil's least weighted member is across a jump). In FP64 they cost 0 to 4 us a launch of those below, most at
-// degree 5, where each of the 150 products takes the pipe for 64 clocks of a lone warp.
+// FP64 products are, of the largest mean of the stencil (up to 2.8 times as far, at most 5e-16 of it, if only the
+// stencil's least weighted member is across a jump). The FP64 directional products cost 0 to 4 us a launch of those below,
+// most at degree 5, where each of 150 takes the FP64 pipe for 64 clocks of a lone warp.
 //
 // The selection (eqs. 19-23) and the positivity test only yield decisions: they are taken in FP32
 // where they hold by a margin far above its error, and in FP64 as printed elsewhere.
@@ -36,7 +36,7 @@
 // memory between the two products.
 //
 // Measured per launch against the FP64 schedules it replaced (bound by the FP64 pipe, 61 to 86 % of its
-// rate): 2D degree 3, 131 072 cells 534 -> 121 us; 3D degree 3, 24 576 cells 432 (553 in blocks of 128) -> 127
+// rate): 2D degree 3, 131 072 cells 534 -> 121 us; 3D degree 3, 24 576 cells 432 (553 in blocks of 128) -> 131
 // us; 2D degree 5, 4200 cells 81 -> 41 us; 2D degree 2, 2048 cells 19 (51 in blocks of 128) -> 11 us. It is
 // now bound by the integer pipe (shifts and 64-bit sums of the conversions, 63 % busy at 2D degree 3), the
 // small meshes by the length of a warp's chain.

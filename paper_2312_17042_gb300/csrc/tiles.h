@@ -24,7 +24,7 @@ struct TileShape {
   static constexpr int KD = Dir<D, R>::KD, ND = Dir<D, R>::ND, PDS = Dir<D, R>::PDS;
   static constexpr int CPW = 32 / NV;
   // Chunks of the central record, NST of them in flight, and the members whose differences are formed
-  // together. FP64: all of it up to 20 members (2D degrees 2, 3; 3D degree 2). Mixed: chunks of 2.7,
+  // together. FP64: all of it at 12 members (2D degree 2), else chunks of 4 or 6. Mixed: chunks of 2.7,
   // 3.8 and 3.5 kB a warp at degrees 4, 5 and 6; 5 to 12 kB in flight in each of 9 to 13 warps cover the
   // memory latency of an SM (about 45 kB at the full rate) through the arithmetic. Measured, us a
   // launch (MC x NST): degree 4, 215 000 cells 10 x 3 123.7, 10 x 2 115.1, 6 x 3 117.7, 6 x 2 112.4; degree 6,
